@@ -160,7 +160,7 @@ adam_apply_narrow_kernel(const __grid_constant__ UpdateGroup grp, int64_t ldgc, 
   grid_dep_wait();
   const int lay = blockIdx.z;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int32_t* __restrict__ idx = grp.idx[lay];
+  const int32_t* idx = grp.idx[lay];
   const RowArgs p = {grp.part[lay], grp.Gc[lay], grp.M[lay], grp.V[lay], grp.U[lay], grp.rho[lay],
                      ldgc, ldstate, n, ld_part, split_stride, split_k, part_by_row, reset};
   const int64_t c = static_cast<int64_t>(blockIdx.x) * 32 + lane;
@@ -270,7 +270,7 @@ adam_apply_wide_kernel(const __grid_constant__ UpdateGroup grp, int64_t ldgc, in
   __shared__ float s_scale[kThreads / 32];
   grid_dep_wait();
   const int lay = blockIdx.z, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int32_t* __restrict__ idx = grp.idx[lay];
+  const int32_t* idx = grp.idx[lay];
   const RowArgs p = {grp.part[lay], grp.Gc[lay], grp.M[lay], grp.V[lay], grp.U[lay], grp.rho[lay],
                      ldgc, ldstate, n, ld_part, split_stride, split_k, part_by_row, reset};
   const int j0 = blockIdx.y;
@@ -337,8 +337,8 @@ adam_apply_cols_kernel(const __grid_constant__ UpdateGroup grp, int64_t ldgc, in
   __shared__ float s_u[J][33];
   grid_dep_wait();
   const int lay = blockIdx.z, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int32_t* __restrict__ idx = grp.idx[lay];
-  const float* __restrict__ rho = grp.rho[lay];
+  const int32_t* idx = grp.idx[lay];
+  const float* rho = grp.rho[lay];
   const float* part = grp.part[lay];
   float *Gc = grp.Gc[lay], *M = grp.M[lay], *V = grp.V[lay], *U = grp.U[lay];
   // blocks run along j first: those of one moment cover whole rows of W (512-byte pieces of every row

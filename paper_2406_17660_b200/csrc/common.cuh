@@ -52,6 +52,11 @@ struct ProfileScope {
 // and each later kernel waits before it touches memory, so completion is transitive along the chain.
 // A kernel that something follows lets it in with grid_dep_launch(), late enough that the waiting
 // blocks do not hold an SM that another stream could use.
+// What an earlier kernel of the call writes (G_C, partials, norms, idx, rho, the gathered operand) is
+// still being written when a dependent kernel becomes resident, so it is not constant for that kernel's
+// lifetime: such a kernel reads it with ordinary loads (also ptx::ld_s32, ld_f32), through pointers
+// without __restrict__ and without __ldg, which the compiler could move above grid_dep_wait().  Read-only
+// loads (ld_nc_*) are for inputs of the call.
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -563,7 +563,7 @@ project_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
         const int j = col0 + 32 * i + lane;
         int row = -1;
         if (j < p.r) {
-          row = __ldg(idx + j);
+          row = ptx::ld_s32(idx + j);
           if (row < 0 || row >= p.m) {
             record_status(p.status, GRASS_ERR_INVALID_ARG, row);
             row = -1;
@@ -620,7 +620,7 @@ project_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
           const int j = jb + 32 * h + lane;
           int row = -1;
           if (j < p.r) {
-            row = __ldg(idx + j);
+            row = ptx::ld_s32(idx + j);
             if (row < 0 || row >= p.m) {
               record_status(p.status, GRASS_ERR_INVALID_ARG, row);
               row = -1;
@@ -735,7 +735,7 @@ project_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
           continue;
         }
         float my_rho = 1.f;
-        if (scale && row0 + lane < p.r) my_rho = __ldg(rho + row0 + lane);
+        if (scale && row0 + lane < p.r) my_rho = ptx::ld_f32(rho + row0 + lane);
         float* dst = out + static_cast<long long>(row0) * ld + c;
         const int nvalid = p.r - row0 < 32 ? p.r - row0 : 32;
         if (nvalid == 32) {
@@ -792,9 +792,9 @@ gather_cols_kernel(const GatherGroup grp, long long lddy, int T, int m, int r, i
   grid_dep_launch();        // the blocks of the GEMM find room only when the last of these run
   grid_dep_wait();
   // blockIdx.z = layer of the group
-  const __nv_bfloat16* __restrict__ dY = grp.dY[blockIdx.z];
-  const int32_t* __restrict__ idx = grp.idx[blockIdx.z];
-  __nv_bfloat16* __restrict__ Ag = grp.Ag[blockIdx.z];
+  const __nv_bfloat16* dY = grp.dY[blockIdx.z];
+  const int32_t* idx = grp.idx[blockIdx.z];
+  __nv_bfloat16* Ag = grp.Ag[blockIdx.z];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int jb = blockIdx.x * (32 * ni);
   int rows[8];
@@ -803,7 +803,7 @@ gather_cols_kernel(const GatherGroup grp, long long lddy, int T, int m, int r, i
     const int j = jb + 32 * i + lane;
     int row = -1;
     if (i < ni && j < r) {
-      row = __ldg(idx + j);
+      row = ptx::ld_s32(idx + j);
       if (row < 0 || row >= m) {
         record_status(status, GRASS_ERR_INVALID_ARG, row);
         row = -1;
@@ -848,9 +848,9 @@ splitk_reduce_kernel(const ReduceGroup grp, long long ld_part, long long split_s
                      int r, int n, long long ldgc, int vec) {
   grid_dep_wait();
   // blockIdx.y = layer of the group
-  const float* __restrict__ part = grp.part[blockIdx.y];
-  const float* __restrict__ rho = grp.rho[blockIdx.y];
-  float* __restrict__ Gc = grp.Gc[blockIdx.y];
+  const float* part = grp.part[blockIdx.y];
+  const float* rho = grp.rho[blockIdx.y];
+  float* Gc = grp.Gc[blockIdx.y];
   const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
   if (vec) {
     const int nv = n / 4;
@@ -875,7 +875,7 @@ splitk_reduce_kernel(const ReduceGroup grp, long long ld_part, long long split_s
         const float4 v = *reinterpret_cast<const float4*>(src + s * split_stride);
         acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
       }
-      const float sc = rho != nullptr ? __ldg(rho + row) : 1.f;
+      const float sc = rho != nullptr ? rho[row] : 1.f;
       acc.x *= sc; acc.y *= sc; acc.z *= sc; acc.w *= sc;
       *reinterpret_cast<float4*>(Gc + static_cast<long long>(row) * ldgc + col) = acc;
     }
@@ -887,7 +887,7 @@ splitk_reduce_kernel(const ReduceGroup grp, long long ld_part, long long split_s
       const float* src = part + static_cast<long long>(row) * ld_part + col;
       float acc = *src;
       for (int s = 1; s < split_k; ++s) acc += src[s * split_stride];
-      Gc[static_cast<long long>(row) * ldgc + col] = acc * (rho != nullptr ? __ldg(rho + row) : 1.f);
+      Gc[static_cast<long long>(row) * ldgc + col] = acc * (rho != nullptr ? rho[row] : 1.f);
     }
   }
 }
@@ -898,8 +898,8 @@ splitk_reduce_kernel(const ReduceGroup grp, long long ld_part, long long split_s
 // columns past n of the last four are masked out), columns in a fixed thread-strided order, then
 // a shuffle tree and one shared-memory hop: bit-reproducible.
 __global__ void __launch_bounds__(256)
-splitk_rownorms_kernel(const float* __restrict__ part, long long ld_part, long long split_stride,
-                       int split_k, int m, int n, float* __restrict__ norms) {
+splitk_rownorms_kernel(const float* part, long long ld_part, long long split_stride,
+                       int split_k, int m, int n, float* norms) {
   __shared__ float s_part[8];
   grid_dep_launch();
   grid_dep_wait();
@@ -938,8 +938,7 @@ splitk_rownorms_kernel(const float* __restrict__ part, long long ld_part, long l
 
 // norms[j] = sqrt(sum over column groups g of part[g][j]), groups added in increasing g.
 __global__ void __launch_bounds__(256)
-norms_finalize_kernel(const float* __restrict__ part, long long ld, int groups, int m,
-                      float* __restrict__ norms) {
+norms_finalize_kernel(const float* part, long long ld, int groups, int m, float* norms) {
   grid_dep_launch();
   grid_dep_wait();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;

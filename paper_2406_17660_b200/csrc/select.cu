@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(kThreads) select_rank_kernel(SelectArgs a, int
   for (int i0 = tid; i0 < rows; i0 += 4 * kThreads) {
     float v[4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) v[u] = i0 + u * kThreads < rows ? __ldg(a.norms + row0 + i0 + u * kThreads) : 0.f;
+    for (int u = 0; u < 4; ++u) v[u] = i0 + u * kThreads < rows ? a.norms[row0 + i0 + u * kThreads] : 0.f;
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int i = i0 + u * kThreads;
@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(kThreads) select_kernel(SelectArgs a) {
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         const int k = k0 + u * kThreads;
-        v[u] = k < m ? __ldg(a.norms + k) : 0.f;
+        v[u] = k < m ? a.norms[k] : 0.f;
       }
 #pragma unroll
       for (int u = 0; u < 8; ++u) {

@@ -95,6 +95,18 @@ __device__ __forceinline__ int flag_load_acquire(const int* flag) {
 __device__ __forceinline__ void fence_proxy_async_global() {
   asm volatile("fence.proxy.async.global;" ::: "memory");
 }
+// Ordinary loads of what an earlier kernel of the call wrote, after grid_dep_wait().
+__device__ __forceinline__ int ld_s32(const int* p) {
+  int v;
+  asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ float ld_f32(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+  return v;
+}
+
 // 16-bit read-only load that does not allocate in L1 (each selected column is read once).  An L2
 // miss fetches 128 bytes by default; HALF_LINE lowers the prefetch size to 64 bytes, which is what
 // an isolated pick should pay for (16 M isolated 2-byte reads: 276 -> 165 us).
