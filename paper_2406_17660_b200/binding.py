@@ -469,7 +469,7 @@ class LayerStepCall:
         self._ref = ctypes.byref(a)
         self._slots = (a.dY, a.X, a.idx, a.rho, a.Gc, a.M, a.V, a.U, a.W)
         self._launch = load_library().grass_layer_step
-        self._hyper = self._now = None
+        self._now = None
 
     def __reduce__(self):
         return (LayerStepCall, ())       # a copied layer marshals its own buffers anew
@@ -534,9 +534,7 @@ class LayerStepCall:
     def _scalars(self, count, ws, hyper, step):
         a = self.args
         a.count, a.step = count, step
-        if hyper != self._hyper:
-            self._hyper = hyper
-            a.lr, a.beta1, a.beta2, a.eps, a.alpha = hyper
+        a.lr, a.beta1, a.beta2, a.eps, a.alpha = hyper
         a.ws, a.ws_bytes = (None, 0) if ws is None else (ws.data_ptr(), ws.nbytes)
 
     def launch(self, count, ws, lr, beta1, beta2, eps, step, alpha) -> None:
