@@ -478,18 +478,23 @@ class LayerStepCall:
         """Layer g's selection, state and weights; layer 0 sets sizes, pitches and W's dtype.
         cols: idx selects columns of W, whose rows the state runs along."""
         f32 = torch.float32
-        if not (M.dtype is f32 and V.dtype is f32 and Gc.dtype is f32 and idx.dtype is torch.int32):
-            raise TypeError("Gc, M and V must be float32 and idx int32")
-        if not (M.is_cuda and V.is_cuda and Gc.is_cuda and W.is_cuda and idx.is_cuda):
+        if not (M.dtype is f32 and V.dtype is f32 and Gc.dtype is f32 and idx.dtype is torch.int32
+                and (rho is None or rho.dtype is f32) and (U is None or U.dtype is f32)):
+            raise TypeError("Gc, M, V, U and rho must be float32 and idx int32")
+        if not (M.is_cuda and V.is_cuda and Gc.is_cuda and W.is_cuda and idx.is_cuda
+                and (rho is None or rho.is_cuda) and (U is None or U.is_cuda)):
             raise TypeError("a layer step takes CUDA tensors")
         shape, stride, wshape = M.shape, M.stride(), W.shape
         r, n = shape
         k = 1 if cols else 0
-        if V.shape != shape or Gc.shape != shape or wshape[1 - k] != n or idx.shape[0] != r:
-            raise ValueError("Gc, M and V must be r x n, idx r long and W m x n")
+        if V.shape != shape or Gc.shape != shape or wshape[1 - k] != n or (U is not None and U.shape != shape):
+            raise ValueError("Gc, M, V and U must be r x n and W m x n")
+        if idx.numel() < r or not idx.is_contiguous() or \
+                (rho is not None and (rho.numel() < r or not rho.is_contiguous())):
+            raise ValueError("idx and rho must hold one value per selected row, next to one another")
         ldm = _pitch(shape, stride)
         if (V.stride() != stride and _ld(V) != ldm) or \
-                (U is not None and (U.dtype is not f32 or (U.stride() != stride and _ld(U) != ldm))):
+                (U is not None and U.stride() != stride and _ld(U) != ldm):
             raise ValueError("M, V and U must share one row pitch")
         code = _CODES.get(W.dtype)
         if code is None:

@@ -74,3 +74,35 @@ def test_a_hyper_parameter_changed_in_place_reaches_the_next_call(calls):
         alpha *= 2
     assert [c[1]["lr"] for c in calls] == [1e-3, 5e-4]
     assert [c[1]["alpha"] for c in calls] == [0.25, 0.5]
+
+
+@pytest.mark.parametrize("name,bad,error", [
+    ("rho", torch.zeros(R), TypeError),                          # host memory
+    ("rho", gpu(R, dtype=torch.float64), TypeError),
+    ("rho", gpu(R, dtype=torch.bfloat16), TypeError),
+    ("rho", gpu(R - 1), ValueError),
+    ("rho", gpu(2 * R)[::2], ValueError),
+    ("idx", torch.zeros(R, dtype=torch.int32), TypeError),
+    ("idx", gpu(R, dtype=torch.int64), TypeError),
+    ("idx", gpu(R - 1, dtype=torch.int32), ValueError),
+    ("idx", gpu(2 * R, dtype=torch.int32)[::2], ValueError),
+    ("U", torch.zeros(R, N), TypeError),
+    ("U", gpu(R, N, dtype=torch.float64), TypeError),
+    ("U", gpu(R - 1, N), ValueError),
+    ("U", gpu(R, N - 1), ValueError),
+    ("U", gpu(R, N + 8)[:, :N], ValueError),                     # not M's pitch
+    ("M", gpu(R, N + 1), ValueError), ("V", gpu(R - 1, N), ValueError), ("Gc", gpu(R, N, dtype=torch.float64), TypeError),
+    ("W", gpu(M, N, dtype=torch.float16), TypeError), ("W", gpu(M, N + 1), ValueError),
+], ids=lambda v: v if isinstance(v, str) else "")
+def test_a_layers_buffers_are_checked_before_a_call_points_at_them(calls, name, bad, error):
+    with pytest.raises(error):
+        B.LayerStepCall().state(0, **dict(buffers(), **{name: bad}))
+
+
+def test_what_a_layer_may_leave_out_or_have_to_spare(calls):
+    call = B.LayerStepCall()
+    call.state(0, **dict(buffers(), U=None, rho=None))
+    assert call.args.U[0] is None and call.args.rho[0] is None
+    longer = dict(buffers(), idx=gpu(R + 3, dtype=torch.int32), rho=gpu(R + 3))
+    call.state(0, **longer)
+    assert call.args.r == R and call.args.rho[0] == longer["rho"].data_ptr()
