@@ -699,10 +699,27 @@ bool make_keep_plan(int64_t T, int64_t m, int64_t n, int r, TcPlan* plan) {
   return bytes <= kKeepMostBytes && bytes / 3e6 < projection_us(t, T, m, n, r, 1) + 6.0;
 }
 
+// The same where the workspace of the norms has room for the partials.
+bool keeps(int64_t T, int64_t m, int64_t n, int r, size_t ws_bytes, TcPlan* plan) {
+  return make_keep_plan(T, m, n, r, plan) && ws_bytes >= grad_parts_bytes(plan->split_k, m, plan->ld_part);
+}
+bool keeps_fp32(int64_t T, int64_t m, int64_t n, int r, size_t ws_bytes) {
+  return keep_fp32(T, m, n, r) && ws_bytes >= make_fp32_plan(T, n, static_cast<int>(m), r).part_bytes;
+}
+
 // Bytes of workspace a plan needs for `count` layers: [control block][per layer: gathered operand,
 // split-K partials].
 size_t plan_ws_bytes(const TcPlan& plan, int count) {
   return plan.ctrl_bytes + (plan.ag_bytes + plan.part_bytes) * static_cast<size_t>(count);
+}
+
+// What a plan cannot be run with: token counts past the pre-pass' grid or the 16-bit slice table, or a
+// workspace of less than `need` bytes.
+int plan_refused(const TcPlan& plan, int64_t T, size_t need, const void* ws, size_t ws_bytes) {
+  if (plan.gather == kOptPrepass && T > 65535LL * kGatherTokens) return GRASS_ERR_UNSUPPORTED;   // grid.y
+  if (plan.unit_begin[plan.split_k] > 65535) return GRASS_ERR_UNSUPPORTED;
+  if (need > 0 && (ws == nullptr || !aligned_to(ws, 256) || ws_bytes < need)) return GRASS_ERR_WORKSPACE;
+  return GRASS_OK;
 }
 
 // Projection of `count` same-shaped layers in one set of launches (count = 1 for the plain
@@ -726,20 +743,15 @@ int project_bf16(int count, const void* const* dY, int64_t lddy, const void* con
   }
   TcPlan plan;
   // kept for G_C (stored even where the tokens are not split), if there is room for it
-  const bool stored = keep != nullptr && make_keep_plan(T, m, n, keep->r, &plan) &&
-                      ws_bytes >= grad_parts_bytes(plan.split_k, m, plan.ld_part);
+  const bool stored = keep != nullptr && keeps(T, m, n, keep->r, ws_bytes, &plan);
   if (!stored)
     plan = norms != nullptr ? make_norms_plan(T, m, n) : make_plan(T, m, n, r, gather, opts, false, count);
-  if (plan.gather == kOptPrepass && T > 65535LL * kGatherTokens)
-    return GRASS_ERR_UNSUPPORTED;                                            // pre-pass grid.y
-  if (plan.unit_begin[plan.split_k] > 65535) return GRASS_ERR_UNSUPPORTED;   // 16-bit slice table
   const bool fused_norms = norms != nullptr && plan.split_k == 1 && !stored;
   const size_t per_layer = fused_norms ? norm_part_bytes(m, n)
                            : stored    ? grad_parts_bytes(plan.split_k, m, plan.ld_part)
                                        : plan.ag_bytes + plan.part_bytes;
-  const size_t need = plan.ctrl_bytes + per_layer * count;
-  if (need > 0 && (ws == nullptr || !aligned_to(ws, 256) || ws_bytes < need))
-    return GRASS_ERR_WORKSPACE;
+  const int refused = plan_refused(plan, T, plan.ctrl_bytes + per_layer * count, ws, ws_bytes);
+  if (refused != GRASS_OK) return refused;
   cudaError_t err;
   int* status = status_word(&err);
   if (status == nullptr) GRASS_CUDA_TRY(err);
@@ -1083,6 +1095,21 @@ int project_and_update(const grass_step_t* a, UpdateCall& u, cudaStream_t s, boo
                       nullptr, refresh);
 }
 
+// What the projection of a refresh iteration will refuse, if it has one: asked before the selection
+// replaces the layer's rows.
+int refresh_projection_refused(const grass_step_t* a, size_t norm_ws_bytes) {
+  TcPlan plan;
+  if (a->dt == GRASS_F32) {
+    const Fp32Plan fp = make_fp32_plan(a->T, a->n, a->r, a->r);
+    return fp.split > 1 && !keeps_fp32(a->T, a->m, a->n, a->r, norm_ws_bytes) &&
+                   (a->ws == nullptr || !aligned_to(a->ws, 256) || a->ws_bytes < fp.part_bytes)
+               ? GRASS_ERR_WORKSPACE : GRASS_OK;
+  }
+  if (keeps(a->T, a->m, a->n, a->r, norm_ws_bytes, &plan)) return GRASS_OK;
+  plan = make_plan(a->T, a->m, a->n, a->r, true, PlanOpts());
+  return plan_refused(plan, a->T, plan_ws_bytes(plan, 1), a->ws, a->ws_bytes);
+}
+
 // Row norms of dY^T X; keep (may be NULL) learns where the gradient was formed, if it was.
 int grad_row_norms(const void* dY, int64_t lddy, const void* X, int64_t ldx, int dt, int64_t T, int64_t m,
                    int64_t n, float* norms, void* ws, size_t ws_bytes, cudaStream_t s, GradParts* keep) {
@@ -1097,9 +1124,7 @@ int grad_row_norms(const void* dY, int64_t lddy, const void* X, int64_t ldx, int
   if (ws == nullptr || !aligned_to(ws, 256) ||
       ws_bytes < grass_grad_row_norms_workspace_bytes(T, m, n, dt) - 256)
     return GRASS_ERR_WORKSPACE;
-  if (keep != nullptr && (!keep_fp32(T, m, n, keep->r) ||
-                          ws_bytes < make_fp32_plan(T, n, static_cast<int>(m), keep->r).part_bytes))
-    keep = nullptr;
+  if (keep != nullptr && !keeps_fp32(T, m, n, keep->r, ws_bytes)) keep = nullptr;
   const long long ld = static_cast<long long>(round_up(static_cast<size_t>(n), 4));
   return project_fp32(dY, lddy, X, ldx, T, m, n, nullptr, nullptr, static_cast<int32_t>(m),
                       static_cast<float*>(ws), ld, ws, ws_bytes, s, nullptr, norms, keep,
@@ -1149,10 +1174,12 @@ extern "C" int grass_refresh_step(const grass_step_t* a, const grass_refresh_t* 
       (f->select_ws == nullptr || !aligned_to(f->select_ws, 256) ||
        f->select_ws_bytes < grass_select_workspace_bytes(a->m, a->r, f->method)))
     return GRASS_ERR_WORKSPACE;
+  int rc2 = refresh_projection_refused(a, f->norm_ws_bytes);
+  if (rc2 != GRASS_OK) return rc2;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   GradParts kept;
   kept.r = a->r;
-  int rc2 = grad_row_norms(a->dY[0], a->lddy, a->X[0], a->ldx, a->dt, a->T, a->m, a->n, f->norms,
+  rc2 = grad_row_norms(a->dY[0], a->lddy, a->X[0], a->ldx, a->dt, a->T, a->m, a->n, f->norms,
                            f->norm_ws, f->norm_ws_bytes, s, &kept);
   if (rc2 != GRASS_OK) return rc2;
   rc2 = select_rows(true, f->norms, a->m, a->r, f->method, f->seed, f->layer_id, f->epoch,

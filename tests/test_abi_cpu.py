@@ -102,6 +102,23 @@ def test_projection_options_and_limits_are_checked_on_the_host(lib):
         == binding.GATHER_COOPERATIVE
 
 
+@pytest.mark.parametrize("dt,T,m,n,r", [(binding.BF16, 4096, 4096, 4096, 512), (binding.F32, 4096, 4096, 2048, 64)])
+def test_a_refresh_that_cannot_project_is_refused_before_it_selects(lib, dt, T, m, n, r):
+    """Too small or no projection workspace: an error, not new rows with the old state and weights.
+    (Without a device, anything past the argument checks would be a CUDA error.)"""
+    fake = 0x10000                          # never dereferenced
+    step = binding.LayerStep(count=1, dt=dt, wdt=dt, r=r, T=T, m=m, n=n, lddy=m, ldx=n, ldgc=n, ldstate=n, ldw=n,
+                             lr=1e-3, beta1=0.9, beta2=0.999, eps=1e-8, alpha=0.25, step=1)
+    for field in ("dY", "X", "idx", "rho", "Gc", "M", "V", "W"):
+        getattr(step, field)[0] = fake
+    norms = binding.grass_grad_row_norms_workspace_bytes(T, m, n, dt)
+    refresh = binding.Refresh(norms=fake, norm_ws=fake, norm_ws_bytes=norms)
+    assert not binding.grass_refresh_keeps_gradient(T, m, n, r, dt)
+    for ws, nbytes in ((None, 0), (fake, 4096), (fake + 64, 1 << 40)):
+        step.ws, step.ws_bytes = ws, nbytes
+        assert lib.grass_refresh_step(ctypes.byref(step), ctypes.byref(refresh), None) == 5
+
+
 def test_workspace_queries_are_host_only_and_monotone(lib):
     assert binding.grass_select_workspace_bytes(4096, 256, binding.SEL_TOPR) >= 256
     a = binding.grass_select_workspace_bytes(4096, 256, binding.SEL_MULTINOMIAL_NORM)
