@@ -134,9 +134,14 @@ class GrassLayerGroup:
         nbytes = B.grass_project_batched_workspace_bytes(len(layers), T, first.m, first.n, first.r)
         self.ws = torch.empty(nbytes, dtype=torch.uint8, device=device)
         self.stream = None
-        self._call = B.LayerStepCall()      # the layers' own buffers are marshalled once
-        for g, l in enumerate(layers):
-            self._call.state(g, l.idx, l.rho, l.Gc, l.M, l.V, l.U if l.keep_U else None, l.W)
+        self._call = B.LayerStepCall()
+        self._marshal()                     # layers that do not go together are refused here
+
+    def _marshal(self):
+        """The buffers that the layers have now: a layer may have been given others since the last step."""
+        state = self._call.state
+        for g, l in enumerate(self.layers):
+            state(g, l.idx, l.rho, l.Gc, l.M, l.V, l.U if l.keep_U else None, l.W)
 
     def step(self, dYs, Xs):
         ls = self.layers
@@ -150,6 +155,7 @@ class GrassLayerGroup:
                 return
             for l, dY, X in zip(ls, dYs, Xs):
                 l.refresh(dY, X)
+        self._marshal()
         inputs = self._call.inputs
         for g, l in enumerate(ls):
             l.adam_step += 1

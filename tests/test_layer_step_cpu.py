@@ -15,9 +15,16 @@ class OnGpu(torch.Tensor):
     """A host tensor that answers as a CUDA tensor does."""
     is_cuda = True
 
+    def __deepcopy__(self, memo):
+        return memo.setdefault(id(self), self.clone().as_subclass(OnGpu))
+
 
 def gpu(*shape, dtype=torch.float32):
     return torch.zeros(shape, dtype=dtype).as_subclass(OnGpu)
+
+
+LAUNCHING = ("grass_grad_row_norms", "grass_select", "grass_project_grad", "grass_project_grad_batched",
+             "grass_adam_scatter_batched")
 
 
 @pytest.fixture
@@ -45,6 +52,8 @@ def calls(monkeypatch):
         grass_refresh_step = staticmethod(refresh_step)
 
         def __getattr__(self, name):
+            if name in LAUNCHING:
+                return lambda *args: seen.append((name, args, None)) or 0
             return getattr(real, name)
 
     library = Library()
@@ -106,3 +115,41 @@ def test_what_a_layer_may_leave_out_or_have_to_spare(calls):
     longer = dict(buffers(), idx=gpu(R + 3, dtype=torch.int32), rho=gpu(R + 3))
     call.state(0, **longer)
     assert call.args.r == R and call.args.rho[0] == longer["rho"].data_ptr()
+
+
+def layer(m=M, n=N, r=R, tokens=T, K=2, t=0, **kw):
+    W = gpu(m, n, dtype=torch.bfloat16)
+    ws = grass.step.GrassWorkspace([(m, n)], tokens, r, torch.bfloat16, grass.SEL_TOPR, device="cpu")
+    ws.norms = ws.norms.as_subclass(OnGpu)
+    kw = dict(dict(alpha=0.25, lr=1e-3), **kw)
+    l = grass.GrassLayer(W, r, grass.SEL_TOPR, K, workspace=ws, **kw)
+    for name in ("idx", "rho", "Gc", "M", "V", "U"):
+        setattr(l, name, getattr(l, name).as_subclass(OnGpu))
+    l.t = t
+    return l
+
+
+def bf16(count, *shape):
+    return [gpu(*shape, dtype=torch.bfloat16) for _ in range(count)]
+
+
+def test_a_group_steps_the_tensors_that_its_layers_have_now(calls):
+    """A layer whose state or weights were replaced (a checkpoint loaded) after the group was made."""
+    group = grass.step.GrassLayerGroup([layer(t=1), layer(t=1)], T, device="cpu")
+    group.step(bf16(2, T, M), bf16(2, T, N))
+    second = group.layers[1]
+    for name in ("idx", "rho", "Gc", "M", "V", "U", "W"):
+        setattr(second, name, getattr(second, name).clone().as_subclass(OnGpu))
+        second.t = group.layers[0].t = 1
+        group.step(bf16(2, T, M), bf16(2, T, N))
+        assert calls[-1][1][name][1] == getattr(second, name).data_ptr(), name
+        assert calls[-1][1][name][0] == getattr(group.layers[0], name).data_ptr()
+
+
+def test_a_copied_group_steps_its_own_layers(calls):
+    import copy
+    group = grass.step.GrassLayerGroup([layer(t=1), layer(t=1)], T, device="cpu")
+    other = copy.deepcopy(group)
+    other.step(bf16(2, T, M), bf16(2, T, N))
+    for g in range(2):
+        assert calls[-1][1]["W"][g] == other.layers[g].W.data_ptr() != group.layers[g].W.data_ptr()
