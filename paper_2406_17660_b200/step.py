@@ -82,26 +82,34 @@ class GrassLayer:
             self.V.zero_()
             self.adam_step = 0
 
+    def _marshal(self, dY, X):
+        """The layer's call with its buffers and these inputs filled in."""
+        if self._call is None:
+            self._call = B.LayerStepCall()
+        self._call.state(0, self.idx, self.rho, self.Gc, self.M, self.V, self.U if self.keep_U else None,
+                         self.W, self.side == "cols")
+        self._call.inputs(0, dY, X)
+        return self._call
+
+    def _refresh_step(self, dY, X, of, step):
+        """A refresh iteration in one call, with the hyper-parameters of layer `of`."""
+        ws = self.ws
+        self._marshal(dY, X).refresh(ws.project_ws, of.lr, of.beta1, of.beta2, of.eps, step, of.alpha,
+                                     self.method, self.seed, self.layer_id, self.t // self.K,
+                                     self.reset_state, ws.norms, ws.norm_ws, ws.select_ws)
+
     def step(self, dY, X):
         """One iteration of Algorithm 1 for this layer; dY (T x m), X (T x n) on the device."""
         if self.side == "cols":
             dY, X = X, dY        # select columns of X, contract with dY: G_C^T = P^T (X^T dY)
         if self.fused_update:
-            if self._call is None:
-                self._call = B.LayerStepCall()
-            call, ws = self._call, self.ws
-            call.state(0, self.idx, self.rho, self.Gc, self.M, self.V, self.U if self.keep_U else None,
-                       self.W, self.side == "cols")
-            call.inputs(0, dY, X)
             if self.t % self.K == 0:
                 if self.reset_state:
                     self.adam_step = 0
-                call.refresh(ws.project_ws, self.lr, self.beta1, self.beta2, self.eps, self.adam_step + 1,
-                             self.alpha, self.method, self.seed, self.layer_id, self.t // self.K,
-                             self.reset_state, ws.norms, ws.norm_ws, ws.select_ws)
+                self._refresh_step(dY, X, self, self.adam_step + 1)
             else:
-                call.launch(1, ws.project_ws, self.lr, self.beta1, self.beta2, self.eps,
-                            self.adam_step + 1, self.alpha)
+                self._marshal(dY, X).launch(1, self.ws.project_ws, self.lr, self.beta1, self.beta2, self.eps,
+                                            self.adam_step + 1, self.alpha)
             self.adam_step += 1
             self.t += 1
             return
@@ -121,7 +129,8 @@ class GrassLayer:
 class GrassLayerGroup:
     """Up to 8 layers of one shape (row selection, bf16) stepped together: their projections
     run as one set of launches and so do their Adam + apply updates.  The layers keep their
-    own selection, state and weights; rows are re-selected layer by layer."""
+    own selection, state and weights; rows are re-selected layer by layer.  The iteration, lr, betas,
+    eps, alpha and the step count of Adam are those of layer 0, on every iteration."""
 
     def __init__(self, layers, T, device="cuda"):
         if not 1 <= len(layers) <= 8:
@@ -146,20 +155,25 @@ class GrassLayerGroup:
     def step(self, dYs, Xs):
         ls = self.layers
         first = ls[0]
-        if first.t % first.K == 0:
-            if all(l.fused_update for l in ls) and B.grass_refresh_keeps_gradient(
-                    dYs[0].shape[0], first.m, first.n, first.r, B.BF16):
-                # the dense gradient that the norms need already holds the selected rows
-                for l, dY, X in zip(ls, dYs, Xs):
-                    l.step(dY, X)
-                return
-            for l, dY, X in zip(ls, dYs, Xs):
-                l.refresh(dY, X)
         self._marshal()
-        inputs = self._call.inputs
-        for g, l in enumerate(ls):
+        for g in range(len(ls)):
+            self._call.inputs(g, dYs[g], Xs[g])
+        kept = False
+        if first.t % first.K == 0:
+            # the dense gradient that the norms need may already hold the selected rows
+            kept = all(l.fused_update for l in ls) and B.grass_refresh_keeps_gradient(
+                dYs[0].shape[0], first.m, first.n, first.r, B.BF16)
+            for l, dY, X in zip(ls, dYs, Xs):
+                if not kept:
+                    l.refresh(dY, X)
+                elif l.reset_state:
+                    l.adam_step = 0
+        step = first.adam_step + 1
+        if kept:
+            for l, dY, X in zip(ls, dYs, Xs):
+                l._refresh_step(dY, X, first, step)
+        else:
+            self._call.launch(len(ls), self.ws, first.lr, first.beta1, first.beta2, first.eps, step, first.alpha)
+        for l in ls:
             l.adam_step += 1
             l.t += 1
-            inputs(g, dYs[g], Xs[g])
-        self._call.launch(len(ls), self.ws, first.lr, first.beta1, first.beta2, first.eps,
-                          first.adam_step, first.alpha)

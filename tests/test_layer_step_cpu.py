@@ -153,3 +153,37 @@ def test_a_copied_group_steps_its_own_layers(calls):
     other.step(bf16(2, T, M), bf16(2, T, N))
     for g in range(2):
         assert calls[-1][1]["W"][g] == other.layers[g].W.data_ptr() != group.layers[g].W.data_ptr()
+
+
+KEPT, NOT_KEPT = dict(m=M, n=N, r=R, tokens=T), dict(m=4096, n=4096, r=R, tokens=256)
+
+
+@pytest.mark.parametrize("shape", [KEPT, NOT_KEPT], ids=["kept", "not kept"])
+@pytest.mark.parametrize("reset", [True, False])
+def test_a_group_has_one_set_of_hyper_parameters_on_every_path(calls, shape, reset):
+    """Layer 0's lr, betas, eps, alpha and step count go for the group, on a refresh of either kind as on
+    a regular step; each layer keeps its own counters, epoch, layer id and reset flag."""
+    assert B.grass_refresh_keeps_gradient(shape["tokens"], shape["m"], shape["n"], R, B.BF16) == (shape is KEPT)
+    layers = [layer(**shape, lr=1e-3 * (g + 1), alpha=0.25 * (g + 1), beta1=0.9 - g / 10, eps=1e-8 * (g + 1),
+                    layer_id=7 + g, reset_state=reset if g == 0 else not reset) for g in range(2)]
+    for g, l in enumerate(layers):
+        l.t, l.adam_step = 4 + 2 * g, 10 + g
+    group = grass.step.GrassLayerGroup(layers, shape["tokens"], device="cpu")
+    dYs, Xs = bf16(2, shape["tokens"], shape["m"]), bf16(2, shape["tokens"], shape["n"])
+    group.step(dYs, Xs)
+    first = 1 if reset else 11
+    assert [l.adam_step for l in layers] == [first, 12 if reset else 1] and [l.t for l in layers] == [5, 7]
+    if shape is KEPT:
+        assert [c[0] for c in calls] == ["refresh", "refresh"]
+        assert [(c[2]["layer_id"], c[2]["epoch"], bool(c[2]["reset_state"])) for c in calls] == \
+            [(7, 2, reset), (8, 3, not reset)]
+        assert [c[1]["W"][0] for c in calls] == [l.W.data_ptr() for l in layers]
+        got = [(c[1]["lr"], c[1]["beta1"], c[1]["eps"], c[1]["alpha"], c[1]["step"]) for c in calls]
+    else:
+        assert [c[0] for c in calls[:4]] == ["grass_grad_row_norms", "grass_select"] * 2
+        assert [c[1][5:7] for c in calls[1:4:2]] == [(7, 2), (8, 3)]
+        got = [(c[1]["lr"], c[1]["beta1"], c[1]["eps"], c[1]["alpha"], c[1]["step"]) for c in calls[4:]]
+    assert set(got) == {(1e-3, 0.9, 1e-8, 0.25, first)}
+    group.step(dYs, Xs)
+    assert calls[-1][0] == "step" and calls[-1][1]["count"] == 2
+    assert (calls[-1][1]["lr"], calls[-1][1]["alpha"], calls[-1][1]["step"]) == (1e-3, 0.25, first + 1)
