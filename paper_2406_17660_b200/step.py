@@ -158,8 +158,8 @@ class GrassLayerGroup:
         self._marshal()
         for g in range(len(ls)):
             self._call.inputs(g, dYs[g], Xs[g])
-        kept = False
-        if first.t % first.K == 0:
+        refresh, kept = first.t % first.K == 0, False
+        if refresh:
             # the dense gradient that the norms need may already hold the selected rows
             kept = all(l.fused_update for l in ls) and B.grass_refresh_keeps_gradient(
                 dYs[0].shape[0], first.m, first.n, first.r, B.BF16)
@@ -172,6 +172,13 @@ class GrassLayerGroup:
         if kept:
             for l, dY, X in zip(ls, dYs, Xs):
                 l._refresh_step(dY, X, first, step)
+        elif refresh and dYs[0].dtype == torch.bfloat16:
+            # with the token slices, hence the bits, of the projection calls: after a reset they decide signs
+            idxs, rhos, Gcs = [l.idx for l in ls], [l.rho for l in ls], [l.Gc for l in ls]
+            B.grass_project_grad_batched(dYs, Xs, idxs, rhos, first.r, Gcs, self.ws)
+            B.grass_adam_scatter_batched(Gcs, [l.M for l in ls], [l.V for l in ls],
+                                         [l.U if l.keep_U else None for l in ls], [l.W for l in ls], idxs, rhos,
+                                         first.lr, first.beta1, first.beta2, first.eps, step, first.alpha)
         else:
             self._call.launch(len(ls), self.ws, first.lr, first.beta1, first.beta2, first.eps, step, first.alpha)
         for l in ls:

@@ -182,7 +182,12 @@ def test_a_group_has_one_set_of_hyper_parameters_on_every_path(calls, shape, res
     else:
         assert [c[0] for c in calls[:4]] == ["grass_grad_row_norms", "grass_select"] * 2
         assert [c[1][5:7] for c in calls[1:4:2]] == [(7, 2), (8, 3)]
-        got = [(c[1]["lr"], c[1]["beta1"], c[1]["eps"], c[1]["alpha"], c[1]["step"]) for c in calls[4:]]
+        # then the projection call, whose token slices a refresh keeps, and the update
+        assert [c[0] for c in calls[4:]] == ["grass_project_grad_batched", "grass_adam_scatter_batched"]
+        assert list(calls[4][1][11]) == [l.Gc.data_ptr() for l in layers]
+        assert list(calls[5][1][7]) == [l.W.data_ptr() for l in layers]
+        lr, beta1, _, eps, step, alpha = calls[5][1][15:21]
+        got = [(lr, beta1, eps, alpha, step)]
     assert set(got) == {(1e-3, 0.9, 1e-8, 0.25, first)}
     group.step(dYs, Xs)
     assert calls[-1][0] == "step" and calls[-1][1]["count"] == 2
