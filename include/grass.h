@@ -269,7 +269,7 @@ int grass_adam_scatter_batched(int32_t count, const float* const* Gc, int64_t ld
  * grass_project_grad) followed by grass_adam_scatter_batched, with the same arguments, checks and
  * errors.  Where the projection is split over the tokens, the update kernel sums the partials
  * itself, so G_C crosses HBM once.  The step may choose another tiling than the projection calls (the
- * one grass_project_plan reports), so G_C agrees with theirs to fp32 summation order; the update of a given
+ * one grass_project_plan reports; its own: grass_step_plan), so G_C agrees with theirs to fp32 summation order; the update of a given
  * G_C is bit-identical.
  *   dt     dtype of dY and X: GRASS_BF16, or GRASS_F32 (count must be 1).  wdt: dtype of W.
  *   side   GRASS_SIDE_ROWS: P selects rows of W (m x n).  GRASS_SIDE_COLS: it selects columns; the
@@ -386,6 +386,9 @@ typedef struct {
 } grass_project_plan_t;
 int grass_project_plan(int32_t count, int64_t T, int64_t m, int64_t n, int32_t r,
                        const grass_project_opts_t* opts, grass_project_plan_t* plan);
+/* The same report for what grass_layer_step does with bf16 operands on a regular iteration (a refresh
+ * projects as grass_project_grad does). */
+int grass_step_plan(int32_t count, int64_t T, int64_t m, int64_t n, int32_t r, grass_project_plan_t* plan);
 int grass_project_grad_ex(int32_t count, const void* const* dY, int64_t lddy,
                           const void* const* X, int64_t ldx, int64_t T, int64_t m, int64_t n,
                           const int32_t* const* idx, const float* const* rho, int32_t r,

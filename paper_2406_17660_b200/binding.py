@@ -329,6 +329,7 @@ class ProjectPlan(ctypes.Structure):
 _SIGNATURES.update({
     "grass_project_plan": (c_int, [c_int32, c_int64, c_int64, c_int64, c_int32,
                                    ctypes.POINTER(ProjectOpts), ctypes.POINTER(ProjectPlan)]),
+    "grass_step_plan": (c_int, [c_int32, c_int64, c_int64, c_int64, c_int32, ctypes.POINTER(ProjectPlan)]),
     "grass_project_grad_ex": (c_int, [c_int32, c_void_p, c_int64, c_void_p, c_int64, c_int64, c_int64,
                                       c_int64, c_void_p, c_void_p, c_int32, c_void_p, c_int64,
                                       c_void_p, c_size_t, ctypes.POINTER(ProjectOpts), c_void_p]),
@@ -348,6 +349,13 @@ def grass_project_plan(count: int, T: int, m: int, n: int, r: int, opts=None) ->
     plan = ProjectPlan()
     _check(load_library().grass_project_plan(count, T, m, n, r, _opts(opts), ctypes.byref(plan)),
            "grass_project_plan")
+    return {name: int(getattr(plan, name)) for name, _ in ProjectPlan._fields_}
+
+
+def grass_step_plan(count: int, T: int, m: int, n: int, r: int) -> dict:
+    """What grass_layer_step does for bf16 layers of this shape on a regular iteration (host only)."""
+    plan = ProjectPlan()
+    _check(load_library().grass_step_plan(count, T, m, n, r, ctypes.byref(plan)), "grass_step_plan")
     return {name: int(getattr(plan, name)) for name, _ in ProjectPlan._fields_}
 
 

@@ -90,6 +90,12 @@ int tiles_along_n(const TileChoice& t, int64_t n) {
   return static_cast<int>((n + cols - 1) / cols);
 }
 
+// A gather mode's and a tile's limit on the tokens of a call: the separate gather's grid.y, and the units of
+// the kernel's 16-bit slice table.
+bool tokens_fit(int gather, int unit, int64_t T) {
+  return (gather != kOptPrepass || T <= 65535LL * kGatherTokens) && (T + unit - 1) / unit <= 65535;
+}
+
 // Slice lengths for s_long equal slices and ss extra SHORT ones.  With N = tiles-per-slice x slices tiles
 // on W workers equal slices leave the last wave partly empty whenever W does not divide N; the
 // R = N_long mod W workers that receive one long tile more than the rest are then finished, and the
@@ -116,7 +122,7 @@ double short_slices(TileChoice& t, int64_t n_out, int W, int U, double c, double
 }
 
 // Estimated microseconds of projecting `groups` layers with this choice, beyond what every choice
-// costs.  The form is what the parts wait for; the constants are fitted to 25 000 timed layer-steps (80
+// costs; 1e299 for more tokens than the choice takes.  The form is what the parts wait for; the constants are fitted to 25 000 timed layer-steps (80
 // shapes of the LLaMA range, T = 600 .. 65536, r = 16 .. 1024, every tile, mode and slice count that
 // exists) and predict the good choices to 7 %.  The choice made is 2 % slower than the best one on
 // average; the rules that this replaces (tiles as wide as TMEM allows, a separate gather only for
@@ -134,6 +140,7 @@ double projection_us(TileChoice& t, int64_t T, int64_t m, int64_t n, int r, int 
   const int tiles_x = tiles_along_n(t, n);
   const int64_t n_out = static_cast<int64_t>(tiles_x) * t.r_blocks * groups;     // tiles per slice
   const int unit = unit_tokens(t);
+  if (!tokens_fit(t.gather, unit, T)) return 1e299;     // the call would refuse it
   const int U = static_cast<int>((T + unit - 1) / unit);
   const double cols = t.mb * 128.0, rows = t.pair ? t.r_cta / 2 : t.r_cta;
   double c = (cols + rows) * (1.092 / 1700);                                     // us per 32 tokens
@@ -713,11 +720,10 @@ size_t plan_ws_bytes(const TcPlan& plan, int count) {
   return plan.ctrl_bytes + (plan.ag_bytes + plan.part_bytes) * static_cast<size_t>(count);
 }
 
-// What a plan cannot be run with: token counts past the pre-pass' grid or the 16-bit slice table, or a
-// workspace of less than `need` bytes.
+// What a plan cannot be run with: more tokens than its gather or its slice table take, or a workspace of
+// less than `need` bytes.
 int plan_refused(const TcPlan& plan, int64_t T, size_t need, const void* ws, size_t ws_bytes) {
-  if (plan.gather == kOptPrepass && T > 65535LL * kGatherTokens) return GRASS_ERR_UNSUPPORTED;   // grid.y
-  if (plan.unit_begin[plan.split_k] > 65535) return GRASS_ERR_UNSUPPORTED;
+  if (!tokens_fit(plan.gather, plan.kb_unit * plan.bk, T)) return GRASS_ERR_UNSUPPORTED;
   if (need > 0 && (ws == nullptr || !aligned_to(ws, 256) || ws_bytes < need)) return GRASS_ERR_WORKSPACE;
   return GRASS_OK;
 }
@@ -1042,6 +1048,16 @@ extern "C" int grass_project_plan(int32_t count, int64_t T, int64_t m, int64_t n
       r > m || T > 0x7fffffffLL || m > 0x7fffffffLL || n > 0x7fffffffLL || !opts_ok(opts))
     return GRASS_ERR_INVALID_ARG;
   describe_plan(make_plan(T, m, n, r, true, to_plan_opts(opts), false, count), count, plan);
+  return GRASS_OK;
+}
+
+extern "C" int grass_step_plan(int32_t count, int64_t T, int64_t m, int64_t n, int32_t r,
+                               grass_project_plan_t* plan) {
+  using namespace grass;
+  if (plan == nullptr || count < 1 || count > kTcMaxGroup || T < 1 || m < 1 || n < 1 || r < 1 ||
+      r > m || T > 0x7fffffffLL || m > 0x7fffffffLL || n > 0x7fffffffLL)
+    return GRASS_ERR_INVALID_ARG;
+  describe_plan(make_plan(T, m, n, r, true, wide_opts(), false, count), count, plan);
   return GRASS_OK;
 }
 

@@ -119,6 +119,17 @@ def test_a_refresh_that_cannot_project_is_refused_before_it_selects(lib, dt, T, 
         assert lib.grass_refresh_step(ctypes.byref(step), ctypes.byref(refresh), None) == 5
 
 
+@pytest.mark.parametrize("m,n,r", [(2048, 512, 512), (4096, 64, 1024), (512, 8, 192), (1024, 2048, 300)])
+def test_a_step_over_millions_of_tokens_plans_a_gather_that_takes_them(lib, m, n, r):
+    """The separate gather and narrow stages end at 2 097 120 tokens, the cooperative gather at
+    8 388 480: the search must not return what the call then refuses."""
+    for T in (2097120, 2097121, 2200000, 8388480):
+        p = binding.grass_step_plan(1, T, m, n, r)
+        unit = 128 if p["gather"] == binding.GATHER_COOPERATIVE else p["tokens_per_stage"]
+        assert p["gather"] != binding.GATHER_PREPASS or T <= 65535 * 32
+        assert (T + unit - 1) // unit <= 65535
+
+
 def test_workspace_queries_are_host_only_and_monotone(lib):
     assert binding.grass_select_workspace_bytes(4096, 256, binding.SEL_TOPR) >= 256
     a = binding.grass_select_workspace_bytes(4096, 256, binding.SEL_MULTINOMIAL_NORM)
