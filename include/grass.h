@@ -280,6 +280,7 @@ int grass_adam_scatter_batched(int32_t count, const float* const* Gc, int64_t ld
  *   ws     at least grass_project_batched_workspace_bytes(count, T, m, n, r) bytes for GRASS_BF16
  *          (count = 1: grass_project_workspace_bytes will do), grass_project_workspace_bytes for
  *          GRASS_F32; 256-byte aligned.
+ *          (sized for more tokens than T: if the step's own tiling needs more, it takes the projection calls').
  * The struct is a HOST object, read before the call returns.
  */
 #define GRASS_MAX_GROUP 8

@@ -752,6 +752,10 @@ int project_bf16(int count, const void* const* dY, int64_t lddy, const void* con
   const bool stored = keep != nullptr && keeps(T, m, n, keep->r, ws_bytes, &plan);
   if (!stored)
     plan = norms != nullptr ? make_norms_plan(T, m, n) : make_plan(T, m, n, r, gather, opts, false, count);
+  // a workspace sized for more tokens may fall short of a step's own tiling for fewer (more slices): then
+  // the tiling of the projection calls
+  if (opts.wide && gather && plan_refused(plan, T, plan_ws_bytes(plan, count), ws, ws_bytes) == GRASS_ERR_WORKSPACE)
+    plan = make_plan(T, m, n, r, true, PlanOpts(), false, count);
   const bool fused_norms = norms != nullptr && plan.split_k == 1 && !stored;
   const size_t per_layer = fused_norms ? norm_part_bytes(m, n)
                            : stored    ? grad_parts_bytes(plan.split_k, m, plan.ld_part)
