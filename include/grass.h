@@ -390,6 +390,8 @@ int grass_project_plan(int32_t count, int64_t T, int64_t m, int64_t n, int32_t r
 /* The same report for what grass_layer_step does with bf16 operands on a regular iteration (a refresh
  * projects as grass_project_grad does). */
 int grass_step_plan(int32_t count, int64_t T, int64_t m, int64_t n, int32_t r, grass_project_plan_t* plan);
+/* How many plans the calling thread has searched for; each thread keeps its last 256. */
+int64_t grass_plan_searches(void);
 int grass_project_grad_ex(int32_t count, const void* const* dY, int64_t lddy,
                           const void* const* X, int64_t ldx, int64_t T, int64_t m, int64_t n,
                           const int32_t* const* idx, const float* const* rho, int32_t r,

@@ -329,6 +329,7 @@ class ProjectPlan(ctypes.Structure):
 _SIGNATURES.update({
     "grass_project_plan": (c_int, [c_int32, c_int64, c_int64, c_int64, c_int32,
                                    ctypes.POINTER(ProjectOpts), ctypes.POINTER(ProjectPlan)]),
+    "grass_plan_searches": (c_int64, []),
     "grass_step_plan": (c_int, [c_int32, c_int64, c_int64, c_int64, c_int32, ctypes.POINTER(ProjectPlan)]),
     "grass_project_grad_ex": (c_int, [c_int32, c_void_p, c_int64, c_void_p, c_int64, c_int64, c_int64,
                                       c_int64, c_void_p, c_void_p, c_int32, c_void_p, c_int64,
@@ -357,6 +358,11 @@ def grass_step_plan(count: int, T: int, m: int, n: int, r: int) -> dict:
     plan = ProjectPlan()
     _check(load_library().grass_step_plan(count, T, m, n, r, ctypes.byref(plan)), "grass_step_plan")
     return {name: int(getattr(plan, name)) for name, _ in ProjectPlan._fields_}
+
+
+def grass_plan_searches() -> int:
+    """How many plans the calling thread has searched for."""
+    return int(load_library().grass_plan_searches())
 
 
 def grass_project_grad_ex(dYs, Xs, idxs, rhos, r, Gcs, ws, opts=None) -> None:

@@ -5,6 +5,9 @@
 #include <math.h>
 #include <string.h>
 
+#include <deque>
+#include <unordered_map>
+
 #include "common.cuh"
 #include "project_simt.cuh"
 #include "project_tc.cuh"
@@ -438,27 +441,43 @@ TcPlan search_plan(int64_t T, int64_t m, int64_t n, int r, bool has_idx, const P
   return p;
 }
 
-// The search costs up to a millisecond of host time and a training loop asks for the same few shapes over
-// and over: each host thread keeps the last plan of every hash bucket.  A plan is a function of
-// the numbers below and of nothing else.
+// A search costs the host tens to hundreds of microseconds and a training loop asks for the same few dozen
+// plans over and over (a block of a model has three shapes; a step, a refresh's norms and its projection have
+// plans of their own).  Each host thread keeps the last kPlans that it searched and forgets the oldest
+// first, so no set of up to kPlans shapes in use loses one.  (A table with one plan per hash bucket lost
+// two of the three shapes of a 350M block to one another: 0.76 ms of searching a block.)  A plan is a
+// function of its key and of nothing else.
+struct PlanKey {
+  int64_t v[12];
+  bool operator==(const PlanKey& o) const { return memcmp(v, o.v, sizeof(v)) == 0; }
+};
+struct PlanKeyHash {
+  size_t operator()(const PlanKey& k) const {
+    uint64_t h = 0;
+    for (int64_t x : k.v) h = (h ^ static_cast<uint64_t>(x)) * 0x9E3779B97F4A7C15ull, h ^= h >> 32;
+    return static_cast<size_t>(h);
+  }
+};
+constexpr size_t kPlans = 256;
+thread_local int64_t plan_searches = 0;
+
 TcPlan make_plan(int64_t T, int64_t m, int64_t n, int r, bool has_idx, const PlanOpts& opts,
                  bool single_split = false, int groups = 1) {
-  struct Entry {
-    int64_t key[12];
-    TcPlan plan;
-  };
-  constexpr int kEntries = 64;
-  static thread_local Entry cache[kEntries];        // zero-initialised: T = 0 matches no call
-  const int64_t key[12] = {T, m, n, r, has_idx, opts.gather, opts.mb, opts.pair, opts.split,
-                           opts.unit_of * 2 + (opts.wide ? 1 : 0), single_split, groups};
-  uint64_t h = 0;
-  for (int64_t k : key) h = (h ^ static_cast<uint64_t>(k)) * 0x9E3779B97F4A7C15ull;
-  Entry& e = cache[h >> 58];
-  if (memcmp(e.key, key, sizeof(key)) != 0) {
-    e.plan = search_plan(T, m, n, r, has_idx, opts, single_split, groups);
-    memcpy(e.key, key, sizeof(key));
+  static thread_local std::unordered_map<PlanKey, TcPlan, PlanKeyHash> plans;
+  static thread_local std::deque<PlanKey> order;
+  const PlanKey key = {{T, m, n, r, has_idx, opts.gather, opts.mb, opts.pair, opts.split,
+                        opts.unit_of * 2 + (opts.wide ? 1 : 0), single_split, groups}};
+  const auto hit = plans.find(key);
+  if (hit != plans.end()) return hit->second;
+  ++plan_searches;
+  const TcPlan plan = search_plan(T, m, n, r, has_idx, opts, single_split, groups);
+  if (plans.size() >= kPlans) {
+    plans.erase(order.front());
+    order.pop_front();
   }
-  return e.plan;
+  plans.emplace(key, plan);
+  order.push_back(key);
+  return plan;
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
@@ -1064,6 +1083,8 @@ extern "C" int grass_step_plan(int32_t count, int64_t T, int64_t m, int64_t n, i
   describe_plan(make_plan(T, m, n, r, true, wide_opts(), false, count), count, plan);
   return GRASS_OK;
 }
+
+extern "C" int64_t grass_plan_searches(void) { return grass::plan_searches; }
 
 extern "C" int grass_project_grad_ex(int32_t count, const void* const* dY, int64_t lddy,
                                      const void* const* X, int64_t ldx, int64_t T, int64_t m,

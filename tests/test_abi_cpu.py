@@ -8,6 +8,7 @@ import pytest
 
 import __graft_entry__ as entry
 from paper_2406_17660_b200 import binding
+from paper_2406_17660_b200 import synthetic as syn
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
@@ -128,6 +129,35 @@ def test_a_step_over_millions_of_tokens_plans_a_gather_that_takes_them(lib, m, n
         unit = 128 if p["gather"] == binding.GATHER_COOPERATIVE else p["tokens_per_stage"]
         assert p["gather"] != binding.GATHER_PREPASS or T <= 65535 * 32
         assert (T + unit - 1) // unit <= 65535
+
+
+@pytest.mark.parametrize("T,r", [(T, r) for T in (512, 2048, 8192, 16384, 32768, 65536) for r in (64, 128, 256, 512, 1024)])
+def test_the_plans_of_a_model_are_searched_for_once(lib, T, r):
+    """Steps, groups and refreshes of all shapes of a block, one after another as a training step walks them:
+    the second walk finds every plan of the first."""
+    def walk(dims):
+        hidden, ffn = dims
+        for count, m, n in ((4, hidden, hidden), (2, ffn, hidden), (1, hidden, ffn)):
+            rr = min(r, m)
+            for c in {1, count}:
+                binding.grass_step_plan(c, T, m, n, rr)
+                binding.grass_project_plan(c, T, m, n, rr)
+            binding.grass_refresh_keeps_gradient(T, m, n, rr, binding.BF16)
+            binding.grass_refresh_workspace_bytes(T, m, n, rr, binding.BF16)
+            binding.grass_project_workspace_bytes(T, m, n, rr, binding.BF16)
+
+    for dims in set(syn.LLAMA_DIMS.values()):
+        walk(dims)
+        before = binding.grass_plan_searches()
+        walk(dims)
+        assert binding.grass_plan_searches() == before
+    # many more shapes than a thread keeps: the last ones are still there
+    for t in range(300):
+        binding.grass_step_plan(1, 256 + t, 64, 64, 16)
+    before = binding.grass_plan_searches()
+    for t in range(200, 300):
+        binding.grass_step_plan(1, 256 + t, 64, 64, 16)
+    assert binding.grass_plan_searches() == before
 
 
 def test_workspace_queries_are_host_only_and_monotone(lib):
