@@ -137,75 +137,134 @@ double short_slices(TileChoice& t, int64_t n_out, int W, int U, double c, double
 //             kernel against both, in the 3-norm: the cooperative one needs 15 us where the separate one needs
 //             1 (eight warps an SM against a full one), and is the better choice only when the rest hides it
 //   around    the separate gather, or the start of the cooperative one; the partials
-double projection_us(TileChoice& t, int64_t T, int64_t m, int64_t n, int r, int groups) {
+//
+// A search tries thousands of choices, most of them slice counts of the same tile, so what the slices do not
+// change is computed once per tile (TileCost), and choices that cannot beat one already priced are left
+// out (least_span, most_span): 113 us a search without, 9 with, the mean of 6000 shapes of the LLaMA range.
+struct Problem {
+  int64_t T, m, n;
+  int r, groups;
+  double picks, lines;       // selected share of dY's columns; share of its lines that are touched
+};
+Problem make_problem(int64_t T, int64_t m, int64_t n, int r, int groups) {
+  Problem q = {T, m, n, r, groups, static_cast<double>(r) / m, 0};
+  q.lines = 1.0 - pow(1.0 - q.picks, sparse_pick(m, r) ? 32 : 64);
+  return q;
+}
+struct TileCost {
+  int W, U;
+  int64_t n_out;             // tiles per slice
+  double c, f, drain;        // us per unit, per tile; drain > 0: hidden behind the next tile's MMAs
+  double hbm, hbm_p, gather, gather_p;     // and their powers in the norms
+  double l2, around, per_slice;
+  bool fits;
+};
+
+double pow_2_5(double x) { return x * x * sqrt(x); }
+
+TileCost tile_cost(const Problem& q, const TileChoice& t) {
   const double MBYTE = 1e-6;
-  const int W = t.pair ? kSmCount / 2 : kSmCount;
+  const int64_t T = q.T, m = q.m, n = q.n;
+  const int r = q.r, groups = q.groups;
+  TileCost k;
+  k.W = t.pair ? kSmCount / 2 : kSmCount;
   const int tiles_x = tiles_along_n(t, n);
-  const int64_t n_out = static_cast<int64_t>(tiles_x) * t.r_blocks * groups;     // tiles per slice
+  k.n_out = static_cast<int64_t>(tiles_x) * t.r_blocks * groups;
   const int unit = unit_tokens(t);
-  if (!tokens_fit(t.gather, unit, T)) return 1e299;     // the call would refuse it
-  const int U = static_cast<int>((T + unit - 1) / unit);
+  k.fits = tokens_fit(t.gather, unit, T);
+  k.U = static_cast<int>((T + unit - 1) / unit);
   const double cols = t.mb * 128.0, rows = t.pair ? t.r_cta / 2 : t.r_cta;
-  double c = (cols + rows) * (1.092 / 1700);                                     // us per 32 tokens
+  k.c = (cols + rows) * (1.092 / 1700);                                          // us per 32 tokens
   const double mma = t.mb * t.r_cta * (t.pair ? 0.22 : 0.17) / 1700;
-  if (mma > c) c = mma;
-  c *= unit / 32.0;
-  const double f = 0.42 + (t.pair ? 2.0 : 0.0) + 4.5 * t.mb * t.r_cta / 512;
-  double span;
-  if (t.s_short == 0) {
-    const double per_worker = static_cast<double>(n_out) * t.s_long / W;
-    const double waves = static_cast<double>((n_out * t.s_long + W - 1) / W);
-    double tile = (U + t.s_long - 1) / t.s_long * c + f;
-    // row-norm epilogue, few tokens: with two accumulator sets the drain of one tile hides behind the
-    // MMAs of the next (stores do not: they meet the next tile's loads in L2)
-    if (t.gather == 0 && t.s_long == 1 && T <= 1536 && t.mb * t.r_cta <= 256 && per_worker > 2) {
-      const double drain = 4.5 * t.mb * t.r_cta / 512;
-      tile = 0.4 + (tile - f > drain ? tile - f : drain);
-    }
-    span = tile * (0.83 * waves + 0.17 * (per_worker > 1 ? per_worker : 1));
-  } else {
-    span = short_slices(t, n_out, W, U, c, f);
-    if (span >= 1e300) return span;
-  }
-  const double picks = static_cast<double>(r) / m;
-  const double lines = 1.0 - pow(1.0 - picks, sparse_pick(m, r) ? 32 : 64);      // share of dY touched
-  const double dy_mb = groups * 2.0 * T * m * lines * MBYTE, x_mb = groups * 2.0 * T * n * MBYTE;
+  if (mma > k.c) k.c = mma;
+  k.c *= unit / 32.0;
+  k.f = 0.42 + (t.pair ? 2.0 : 0.0) + 4.5 * t.mb * t.r_cta / 512;
+  // row-norm epilogue, few tokens: with two accumulator sets the drain of one tile hides behind the
+  // MMAs of the next (stores do not: they meet the next tile's loads in L2)
+  k.drain = t.gather == 0 && T <= 1536 && t.mb * t.r_cta <= 256 ? 4.5 * t.mb * t.r_cta / 512 : 0;
+  const double dy_mb = groups * 2.0 * T * m * q.lines * MBYTE, x_mb = groups * 2.0 * T * n * MBYTE;
   const double ag_mb = groups * 2.0 * T * t.r_cta * t.r_blocks * MBYTE, out_mb = groups * 4.0 * r * n * MBYTE;
   // load-unit time of one pass over the picks, and how many lines a load instruction of 32 spans
   const double lsu = groups * static_cast<double>(T) * t.r_cta * t.r_blocks / kSmCount / 32e3;
-  double per_load = (m < 32 / picks ? m : 32 / picks) / 64;
+  double per_load = (m < 32 / q.picks ? m : 32 / q.picks) / 64;
   per_load = per_load < 1 ? 1 : per_load > 32 ? 32 : per_load;
-  double hbm = x_mb / 6.0, gather = 0, around = 0;
+  k.hbm = x_mb / 6.0;
+  k.gather = k.around = 0;
   if (t.gather == kOptPrepass) {
-    hbm += 1.1 * ag_mb / 6.0;
-    around = 0.5 + pow(pow(lsu * (0.87 + 0.033 * per_load), 2.5) + pow((dy_mb + ag_mb) / 6.6, 2.5), 0.4);
+    k.hbm += 1.1 * ag_mb / 6.0;
+    k.around = 0.5 + pow(pow_2_5(lsu * (0.87 + 0.033 * per_load)) + pow_2_5((dy_mb + ag_mb) / 6.6), 0.4);
   } else if (t.gather == kOptCoop) {
-    hbm += dy_mb / 5.8;
-    gather = lsu * (15.3 + 0.1 * per_load);
-    around = 5.9;
+    k.hbm += dy_mb / 5.8;
+    k.gather = lsu * (15.3 + 0.1 * per_load);
+    k.around = 5.9;
   } else if (t.gather == kOptCta) {
-    hbm += dy_mb / 4.1;
-    gather = 2.7 * tiles_x * lsu;
+    k.hbm += dy_mb / 4.1;
+    k.gather = 2.7 * tiles_x * lsu;
   } else {
-    hbm += dy_mb / 6.0;              // the dense gradient: dY is the operand
+    k.hbm += dy_mb / 6.0;            // the dense gradient: dY is the operand
   }
-  const int s = t.s_long + t.s_short;
-  if (s > 1) around += 1.0 + s * (out_mb / 11.2 + 0.056);
-  const double l2_mb = static_cast<double>(n_out) * (t.pair ? 2 : 1) * T * (cols + rows) * 2 * MBYTE;
-  const double stream = pow(pow(span, 2.5) + pow(hbm, 2.5), 0.4);
-  return cbrt(stream * stream * stream + gather * gather * gather) + 0.0018 * l2_mb + around;
+  k.hbm_p = pow_2_5(k.hbm);
+  k.gather_p = k.gather * k.gather * k.gather;
+  const double l2_mb = static_cast<double>(k.n_out) * (t.pair ? 2 : 1) * T * (cols + rows) * 2 * MBYTE;
+  k.l2 = 0.0018 * l2_mb;
+  k.per_slice = out_mb / 11.2 + 0.056;
+  return k;
+}
+
+int next_slices(int s) { return s + 1 + s / 16; }      // the counts that a search tries
+int max_slices(const TileCost& k) { return k.U < kTcMaxSlices ? k.U : kTcMaxSlices; }
+
+double around_us(const TileCost& k, int slices) {
+  double around = k.around;
+  if (slices > 1) around += 1.0 + slices * k.per_slice;
+  return around;
+}
+
+double projection_us(const TileCost& k, TileChoice& t) {
+  if (!k.fits) return 1e299;                       // the call would refuse it
+  double span;
+  if (t.s_short == 0) {
+    const double per_worker = static_cast<double>(k.n_out) * t.s_long / k.W;
+    const double waves = static_cast<double>((k.n_out * t.s_long + k.W - 1) / k.W);
+    double tile = (k.U + t.s_long - 1) / t.s_long * k.c + k.f;
+    if (k.drain > 0 && t.s_long == 1 && per_worker > 2)
+      tile = 0.4 + (tile - k.f > k.drain ? tile - k.f : k.drain);
+    span = tile * (0.83 * waves + 0.17 * (per_worker > 1 ? per_worker : 1));
+  } else {
+    span = short_slices(t, k.n_out, k.W, k.U, k.c, k.f);
+    if (span >= 1e300) return span;
+  }
+  const double stream = pow(pow_2_5(span) + k.hbm_p, 0.4);
+  return cbrt(stream * stream * stream + k.gather_p) + k.l2 + around_us(k, t.s_long + t.s_short);
+}
+
+// The workers' time of a choice of this tile is at least this: what it is if they all finish together
+// (without the per-tile part where that may hide).
+double least_span(const TileCost& k, int slices) {
+  return static_cast<double>(k.n_out) / k.W * (k.U * k.c + (k.drain > 0 ? 0 : slices * k.f));
+}
+// And beyond this a choice of so many slices, or more, costs more than cap: projection_us solved for the
+// span.  (One part in 10^9 is for the rounding of the powers.)
+double most_span(const TileCost& k, int slices, double cap) {
+  const double stream = cap * (1 + 1e-9) - k.l2 - around_us(k, slices);
+  const double cube = stream * stream * stream - k.gather_p;
+  if (stream <= 0 || cube <= 0) return -1;
+  const double p = pow(cube, 2.5 / 3) * (1 + 1e-9) - k.hbm_p;
+  return p <= 0 ? -1 : pow(p, 0.4) * (1 + 1e-9);
 }
 
 // The cheapest choice for a layer-step: any gather, and the rows cut into more blocks than TMEM requires
 // where that pays (1 x 4096 x 2048 x 1024, r = 512: 31 us with 512-row tiles, 26 with 128).
 TileChoice choose_wide(int64_t T, int64_t m, int64_t n, int r, int groups) {
+  struct Tile { TileChoice t; TileCost k; };
+  const Problem q = make_problem(T, m, n, r, groups);
   const int r64 = static_cast<int>(round_up(static_cast<size_t>(r), 64)) / 64;   // in slabs of 64 rows
   const int rb_min = (r64 + 7) / 8;
   int rb_max = rb_min < 8 ? 8 : rb_min + 4;
   if (rb_max > r64) rb_max = r64;
-  TileChoice best = {};
-  double best_us = 1e301;
-  int tried_slabs = 0;
+  Tile tiles[8 * 3 * 3 * 2];          // row blocks, gathers, n-blocks, pairs
+  int count = 0, tried_slabs = 0;
+  double cap = 1e301;                 // what some choice costs
   for (int rb = rb_min; rb <= rb_max; ++rb) {
     const int slabs = (r64 + rb - 1) / rb;
     if (slabs == tried_slabs) continue;            // the same tile with an empty block more
@@ -225,31 +284,46 @@ TileChoice choose_wide(int64_t T, int64_t m, int64_t n, int r, int groups) {
         for (int pair = slabs % 2 == 0 ? 1 : 0; pair >= 0; --pair) {
           if (pair && n <= static_cast<int64_t>(t.mb) * 128) continue;  // nothing for the second CTA
           t.pair = pair != 0;
-          const int tiles_x = tiles_along_n(t, n);
           // In-CTA gather: every tile picks its own columns, so tiles of at most 128 rows (the load unit
           // keeps up), picks dense enough that a load of 32 spans at most 6 lines, and at most two
           // CTAs (pairs) that share a token slice.
-          if (gather == kOptCta &&
-              (t.r_cta > 128 || tiles_x * t.r_blocks > 2 || static_cast<int64_t>(r) * 12 < m))
+          if (gather == kOptCta && (t.r_cta > 128 || tiles_along_n(t, n) * t.r_blocks > 2 ||
+                                    static_cast<int64_t>(r) * 12 < m))
             continue;
-          const int W = t.pair ? kSmCount / 2 : kSmCount;
-          const int64_t n_out = static_cast<int64_t>(tiles_x) * t.r_blocks * groups;
-          const int unit = unit_tokens(t);
-          const int64_t U = (T + unit - 1) / unit;
-          const int max_s = U < kTcMaxSlices ? static_cast<int>(U) : kTcMaxSlices;
-          for (int sl = 1; sl <= max_s; sl += 1 + sl / 16) {
-            t.s_long = sl;
-            // short slices where they were measured to pay: launches of three or more waves (7B
-            // down, r = 1024: 587 -> 539 us), and the in-CTA gather, where each worker is bound by its
-            // own gather warps (60M q,k,v,o: 179 -> 155 us)
-            const int64_t n_long = n_out * t.s_long;
-            const int max_short = n_long % W == 0 || (n_long / W < 2 && gather != kOptCta) ? 0 : 3;
-            for (t.s_short = 0; t.s_short <= max_short && t.s_long + t.s_short <= max_s; ++t.s_short) {
-              const double us = projection_us(t, T, m, n, r, groups);
-              if (us < best_us) { best_us = us; best = t; }
-            }
+          const TileCost k = tile_cost(q, t);
+          tiles[count++] = {t, k};
+          // one and two full waves of tiles: usually close to the best, so that little else is priced
+          for (int wave = 1; wave <= 2; ++wave) {
+            const int64_t fill = wave * k.W / k.n_out < max_slices(k) ? wave * k.W / k.n_out : max_slices(k);
+            for (t.s_long = 1; next_slices(t.s_long) <= fill;) t.s_long = next_slices(t.s_long);
+            const double us = projection_us(k, t);
+            if (us < cap) cap = us;
           }
         }
+      }
+    }
+  }
+  TileChoice best = {};
+  double best_us = 1e301;
+  for (int i = 0; i < count; ++i) {
+    TileChoice t = tiles[i].t;
+    const TileCost& k = tiles[i].k;
+    double most = 0;
+    int most_at = 0;                                   // most_span of this many slices
+    for (int sl = 1; sl <= max_slices(k); sl = next_slices(sl)) {
+      if (most_at == 0 || sl == 2 || sl >= 2 * most_at) most = most_span(k, most_at = sl, cap);
+      if (least_span(k, sl) > most) break;             // and more slices cost more
+      t.s_long = sl;
+      // short slices where they were measured to pay: launches of three or more waves (7B
+      // down, r = 1024: 587 -> 539 us), and the in-CTA gather, where each worker is bound by its
+      // own gather warps (60M q,k,v,o: 179 -> 155 us)
+      const int64_t n_long = k.n_out * t.s_long;
+      const int max_short = n_long % k.W == 0 || (n_long / k.W < 2 && t.gather != kOptCta) ? 0 : 3;
+      for (t.s_short = 0; t.s_short <= max_short && t.s_long + t.s_short <= max_slices(k); ++t.s_short) {
+        if (least_span(k, t.s_long + t.s_short) > most) break;
+        const double us = projection_us(k, t);
+        if (us < best_us) { best_us = us; best = t; }
+        if (us < cap) cap = us;
       }
     }
   }
@@ -355,6 +429,7 @@ TileChoice choose_by_clocks(int64_t T, int64_t m, int64_t n, int r, bool has_idx
 // 189 us with 512 rows, 166 with 256; 3584 x 13824 x 1024: 88, 74 with 384; 3328 x 1376 x 4096: 48, 41 with 192).
 TileChoice choose_dense(int64_t T, int64_t m, int64_t n, const PlanOpts& opts, bool single_split) {
   const int r64 = static_cast<int>(round_up(static_cast<size_t>(m), 64)) / 64;
+  const Problem q = make_problem(T, m, n, static_cast<int>(m), 1);
   TileChoice best = {};
   double best_us = 1e301;
   for (int want = r64 < 8 ? r64 : 8; want >= 1; --want) {
@@ -367,13 +442,15 @@ TileChoice choose_dense(int64_t T, int64_t m, int64_t n, const PlanOpts& opts, b
       for (int pair = slabs % 2 == 0 ? 1 : 0; pair >= 0; --pair) {
         if (pair && n <= static_cast<int64_t>(t.mb) * 128) continue;  // nothing for the second CTA
         t.pair = pair != 0;
-        const int unit = unit_tokens(t);
-        if (opts.unit_of > 0 && opts.unit_of % unit != 0) continue;
-        const int64_t U = (T + unit - 1) / unit;
-        const int max_s = single_split ? 1 : (U < kTcMaxSlices ? static_cast<int>(U) : kTcMaxSlices);
-        for (int sl = 1; sl <= max_s; sl += 1 + sl / 16) {
+        if (opts.unit_of > 0 && opts.unit_of % unit_tokens(t) != 0) continue;
+        const TileCost k = tile_cost(q, t);
+        const int max_s = single_split ? 1 : max_slices(k);
+        double most = 0;
+        for (int sl = 1; sl <= max_s; sl = next_slices(sl)) {
           t.s_long = opts.split > 0 ? (opts.split < max_s ? opts.split : max_s) : sl;
-          const double us = projection_us(t, T, m, n, static_cast<int>(m), 1);
+          if (sl == 2) most = most_span(k, sl, best_us);
+          if (sl >= 2 && least_span(k, sl) > most) break;
+          const double us = projection_us(k, t);
           if (us < best_us) { best_us = us; best = t; }
           if (opts.split > 0) break;
         }
@@ -383,7 +460,7 @@ TileChoice choose_dense(int64_t T, int64_t m, int64_t n, const PlanOpts& opts, b
   // the tile as large as TMEM allows stays unless another is better by more than the model is sure of
   TileChoice large = choose_by_clocks(T, m, n, static_cast<int>(m), false, opts, single_split, 1);
   if (opts.unit_of > 0 && opts.unit_of % unit_tokens(large) != 0) return best;
-  return projection_us(large, T, m, n, static_cast<int>(m), 1) < 1.06 * best_us ? large : best;
+  return projection_us(tile_cost(q, large), large) < 1.06 * best_us ? large : best;
 }
 
 // The result depends only on the arguments.
@@ -441,7 +518,7 @@ TcPlan search_plan(int64_t T, int64_t m, int64_t n, int r, bool has_idx, const P
   return p;
 }
 
-// A search costs the host tens to hundreds of microseconds and a training loop asks for the same few dozen
+// A search costs the host ten to a hundred microseconds and a training loop asks for the same few dozen
 // plans over and over (a block of a model has three shapes; a step, a refresh's norms and its projection have
 // plans of their own).  Each host thread keeps the last kPlans that it searched and forgets the oldest
 // first, so no set of up to kPlans shapes in use loses one.  (A table with one plan per hash bucket lost
@@ -722,7 +799,7 @@ bool make_keep_plan(int64_t T, int64_t m, int64_t n, int r, TcPlan* plan) {
   for (int z = 0; z <= kTcMaxSlices; ++z) plan->unit_begin[z] = proj.unit_begin[z];
   const double bytes = static_cast<double>(grad_parts_bytes(plan->split_k, m, plan->ld_part));
   TileChoice t = {proj.gather, proj.r_cta, proj.r_blocks, proj.MB, proj.pair, proj.split_k, 0, 0};
-  return bytes <= kKeepMostBytes && bytes / 3e6 < projection_us(t, T, m, n, r, 1) + 6.0;
+  return bytes <= kKeepMostBytes && bytes / 3e6 < projection_us(tile_cost(make_problem(T, m, n, r, 1), t), t) + 6.0;
 }
 
 // The same where the workspace of the norms has room for the partials.

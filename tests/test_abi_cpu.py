@@ -3,6 +3,7 @@ symbol include/grass.h declares, and rejects bad arguments before touching the d
 import ctypes
 import os
 import re
+import time
 
 import pytest
 
@@ -158,6 +159,22 @@ def test_the_plans_of_a_model_are_searched_for_once(lib, T, r):
     for t in range(200, 300):
         binding.grass_step_plan(1, 256 + t, 64, 64, 16)
     assert binding.grass_plan_searches() == before
+
+
+def test_a_plan_for_a_new_token_count_costs_little_host_time(lib):
+    """Packed batches bring a new token count every step: the search runs on the host before the launch.
+    The mean over these shapes was 450 us when every choice was priced and is 23; the best of five
+    rounds, each with token counts of its own, has to be below 120."""
+    best = 1e9
+    for attempt in range(5):
+        start, count = time.perf_counter(), 0
+        for hidden, ffn in set(syn.LLAMA_DIMS.values()):
+            for layers, m, n in ((4, hidden, hidden), (2, ffn, hidden), (1, hidden, ffn)):
+                for T, r in ((2048, 128), (16384, 256), (65536, 512)):
+                    binding.grass_step_plan(layers, T - 1 - attempt, m, n, r)
+                    count += 1
+        best = min(best, (time.perf_counter() - start) / count)
+    assert best < 120e-6
 
 
 def test_workspace_queries_are_host_only_and_monotone(lib):
