@@ -82,6 +82,10 @@ class GrassLayer:
             self.V.zero_()
             self.adam_step = 0
 
+    def _own_refresh(self):
+        """Whether a program has put its own in the place of refresh(): then it is that which is called."""
+        return type(self).refresh is not GrassLayer.refresh or "refresh" in self.__dict__
+
     def _marshal(self, dY, X):
         """The layer's call with its buffers and these inputs filled in."""
         if self._call is None:
@@ -102,8 +106,9 @@ class GrassLayer:
         """One iteration of Algorithm 1 for this layer; dY (T x m), X (T x n) on the device."""
         if self.side == "cols":
             dY, X = X, dY        # select columns of X, contract with dY: G_C^T = P^T (X^T dY)
-        if self.fused_update:
-            if self.t % self.K == 0:
+        refresh = self.t % self.K == 0
+        if self.fused_update and not (refresh and self._own_refresh()):
+            if refresh:
                 if self.reset_state:
                     self.adam_step = 0
                 self._refresh_step(dY, X, self, self.adam_step + 1)
@@ -113,7 +118,7 @@ class GrassLayer:
             self.adam_step += 1
             self.t += 1
             return
-        if self.t % self.K == 0:
+        if refresh:
             self.refresh(dY, X)
         self.adam_step += 1
         B.grass_project_grad(dY, X, self.idx, self.rho, self.r, self.Gc, self.ws.project_ws)
@@ -161,7 +166,7 @@ class GrassLayerGroup:
         refresh, kept = first.t % first.K == 0, False
         if refresh:
             # the dense gradient that the norms need may already hold the selected rows
-            kept = all(l.fused_update for l in ls) and B.grass_refresh_keeps_gradient(
+            kept = all(l.fused_update and not l._own_refresh() for l in ls) and B.grass_refresh_keeps_gradient(
                 dYs[0].shape[0], first.m, first.n, first.r, B.BF16)
             for l, dY, X in zip(ls, dYs, Xs):
                 if not kept:

@@ -24,7 +24,7 @@ def gpu(*shape, dtype=torch.float32):
 
 
 LAUNCHING = ("grass_grad_row_norms", "grass_select", "grass_project_grad", "grass_project_grad_batched",
-             "grass_adam_scatter_batched")
+             "grass_adam_scatter_batched", "grass_subspace_adam", "grass_scatter_update", "grass_scatter_update_cols")
 
 
 @pytest.fixture
@@ -117,12 +117,12 @@ def test_what_a_layer_may_leave_out_or_have_to_spare(calls):
     assert call.args.r == R and call.args.rho[0] == longer["rho"].data_ptr()
 
 
-def layer(m=M, n=N, r=R, tokens=T, K=2, t=0, **kw):
+def layer(m=M, n=N, r=R, tokens=T, K=2, t=0, cls=grass.GrassLayer, **kw):
     W = gpu(m, n, dtype=torch.bfloat16)
     ws = grass.step.GrassWorkspace([(m, n)], tokens, r, torch.bfloat16, grass.SEL_TOPR, device="cpu")
     ws.norms = ws.norms.as_subclass(OnGpu)
     kw = dict(dict(alpha=0.25, lr=1e-3), **kw)
-    l = grass.GrassLayer(W, r, grass.SEL_TOPR, K, workspace=ws, **kw)
+    l = cls(W, r, grass.SEL_TOPR, K, workspace=ws, **kw)
     for name in ("idx", "rho", "Gc", "M", "V", "U"):
         setattr(l, name, getattr(l, name).as_subclass(OnGpu))
     l.t = t
@@ -192,3 +192,31 @@ def test_a_group_has_one_set_of_hyper_parameters_on_every_path(calls, shape, res
     group.step(dYs, Xs)
     assert calls[-1][0] == "step" and calls[-1][1]["count"] == 2
     assert (calls[-1][1]["lr"], calls[-1][1]["alpha"], calls[-1][1]["step"]) == (1e-3, 0.25, first + 1)
+
+
+class OwnRows(grass.GrassLayer):
+    """A program's own choice of rows."""
+
+    def refresh(self, dY, X):
+        self.refreshed = (dY, X)
+
+
+@pytest.mark.parametrize("side", ["rows", "cols"])
+def test_a_refresh_of_the_programs_own_is_called(calls, side):
+    l = layer(cls=OwnRows) if side == "rows" else layer(m=N, n=N, cls=OwnRows, side="cols")
+    dY, X = bf16(1, T, M if side == "rows" else N)[0], bf16(1, T, N)[0]
+    l.step(dY, X)
+    assert l.refreshed[0] is (dY if side == "rows" else X)
+    assert [c[0] for c in calls] == ["grass_project_grad", "grass_subspace_adam",
+                                     "grass_scatter_update" if side == "rows" else "grass_scatter_update_cols"]
+    l.step(dY, X)
+    assert calls[-1][0] == "step" and (l.t, l.adam_step) == (2, 2)
+
+
+def test_a_groups_refresh_calls_the_layers_own(calls):
+    layers = [layer(cls=OwnRows), layer(cls=OwnRows)]
+    group = grass.step.GrassLayerGroup(layers, T, device="cpu")
+    dYs, Xs = bf16(2, T, M), bf16(2, T, N)
+    group.step(dYs, Xs)
+    assert [l.refreshed[0] is dY for l, dY in zip(layers, dYs)] == [True, True]
+    assert [c[0] for c in calls] == ["grass_project_grad_batched", "grass_adam_scatter_batched"]
