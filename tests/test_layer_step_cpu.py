@@ -220,3 +220,15 @@ def test_a_groups_refresh_calls_the_layers_own(calls):
     group.step(dYs, Xs)
     assert [l.refreshed[0] is dY for l, dY in zip(layers, dYs)] == [True, True]
     assert [c[0] for c in calls] == ["grass_project_grad_batched", "grass_adam_scatter_batched"]
+
+
+def test_a_single_token_has_no_pitch(calls):
+    """Views of one row differ in a stride that nothing uses; with more rows the layers must agree."""
+    group = grass.step.GrassLayerGroup([layer(t=1), layer(t=1)], T, device="cpu")
+    wide = gpu(4, M + 16, dtype=torch.bfloat16)
+    group.step([wide[:1, :M], bf16(1, 1, M)[0]], [bf16(1, 1, N)[0], gpu(4, N + 8, dtype=torch.bfloat16)[1:2, :N]])
+    assert calls[-1][1]["lddy"] == M + 16 and calls[-1][1]["T"] == 1
+    for bad in ([wide[:2, :M], bf16(1, 2, M)[0]], [wide[:1, :M], bf16(1, 1, M + 1)[0]],
+                [wide[:1, :M], gpu(M, 2, dtype=torch.bfloat16).T[:1]]):
+        with pytest.raises(ValueError):
+            group.step(bad, bf16(2, bad[0].shape[0], N))
