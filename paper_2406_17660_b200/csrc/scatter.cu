@@ -74,7 +74,8 @@ scatter_kernel(T* __restrict__ W, int64_t m, int64_t n, int64_t ldw, const float
 // scaled, and transposed through shared memory; then lane l of a warp owns j = j0 + l, so the
 // 32 lanes touch 32 ascending columns of one W row (few sectors).  The first j of a run of
 // equal columns owns the column and adds the whole run (reaching past the tile through global
-// memory if the run does), so every element is rounded once.
+// memory if the run does), so every element is rounded once.  A term is a product and an add, spelled
+// out: the one-call update (adam_scatter.cu) has the same roundings, hence the same bits.
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
 scatter_cols_kernel(T* __restrict__ W, int64_t m, int64_t n, int64_t ldw,
@@ -88,7 +89,7 @@ scatter_cols_kernel(T* __restrict__ W, int64_t m, int64_t n, int64_t ldw,
     const int j = j0 + jj;
     float v = 0.f;
     if (j < r && c0 + lane < m)
-      v = alpha * (rho != nullptr ? rho[j] : 1.f) * U[static_cast<int64_t>(j) * ldu + c0 + lane];
+      v = __fmul_rn(alpha * (rho != nullptr ? rho[j] : 1.f), U[static_cast<int64_t>(j) * ldu + c0 + lane]);
     tile[jj][lane] = v;
   }
   __syncthreads();
@@ -107,8 +108,9 @@ scatter_cols_kernel(T* __restrict__ W, int64_t m, int64_t n, int64_t ldw,
     if (c >= m) break;
     float acc = 0.f;
     for (int k = 0; k < run; ++k) {
-      if (lane + k < 32) acc += tile[lane + k][cc];
-      else acc += alpha * (rho != nullptr ? rho[j + k] : 1.f) * U[static_cast<int64_t>(j + k) * ldu + c];
+      acc = __fadd_rn(acc, lane + k < 32 ? tile[lane + k][cc]
+                                         : __fmul_rn(alpha * (rho != nullptr ? rho[j + k] : 1.f),
+                                                     U[static_cast<int64_t>(j + k) * ldu + c]));
     }
     T* w = W + c * ldw + col;
     *w = WTraits<T>::add1(*w, acc);

@@ -69,3 +69,28 @@ def test_a_step_over_millions_of_tokens():
     for t in range(0, T, 100_000):
         want += dY[t:t + 100_000, l.idx.long()].double().T @ X[t:t + 100_000].double()
     assert rel(l.Gc, want) <= 1e-4
+
+
+@pytest.mark.parametrize("dtype", [BF16, torch.float32], ids=["bf16", "fp32"])
+@pytest.mark.parametrize("lengths", [(1, 2, 30, 7), (31, 2, 100, 1, 63), (33,), (200,), (5,) * 20])
+def test_the_column_form_rounds_as_the_column_scatter(dtype, lengths):
+    """Columns drawn several times, their runs crossing blocks of 32: the one-call update leaves the same bits
+    as Adam and the column scatter of the same G_C."""
+    T, m, n, r = 256, 300, 77, sum(lengths)
+    rng = np.random.default_rng(r)
+    X, dY = (syn._padded(f(T, k, dtype, seed0=6).to(DEV), syn.pad_to(k, 8))
+             for f, k in ((syn.make_X, m), (syn.make_dY, n)))
+    W0 = syn._padded(syn.make_W(n, m, dtype, seed0=6).to(DEV), syn.pad_to(m, 8))
+    cols = np.repeat(np.sort(rng.choice(m, len(lengths), replace=False)), lengths)
+    ws = grass.step.GrassWorkspace([(m, n)], T, r, dtype, grass.SEL_TOPR)
+    l = grass.GrassLayer(W0.clone(), r, grass.SEL_TOPR, 1 << 30, 0.25, 1e-3, workspace=ws, side="cols")
+    l.idx.copy_(torch.tensor(cols, dtype=torch.int32)); l.t, l.adam_step = 1, 3
+    l.rho.copy_(torch.tensor(0.5 + rng.random(r), dtype=torch.float32))
+    l.M.normal_(); l.V.uniform_(0.5, 1.5)
+    M, V, U, W = l.M.clone(), l.V.clone(), torch.empty_like(l.U), W0.clone()
+    l.step(dY, X)
+    grass.grass_subspace_adam(l.Gc, M, V, U, l.lr, l.beta1, l.beta2, l.eps, 4)
+    grass.grass_scatter_update_cols(W, U, l.idx, l.rho, l.alpha)
+    grass.grass_device_status()
+    for name, want in (("M", M), ("V", V), ("U", U), ("W", W)):
+        assert torch.equal(getattr(l, name), want), name
