@@ -232,3 +232,20 @@ def test_a_single_token_has_no_pitch(calls):
                 [wide[:1, :M], gpu(M, 2, dtype=torch.bfloat16).T[:1]]):
         with pytest.raises(ValueError):
             group.step(bad, bf16(2, bad[0].shape[0], N))
+
+
+def test_a_groups_buffers_are_looked_at_again_after_they_were_refused(calls):
+    group = grass.step.GrassLayerGroup([layer(t=1), layer(t=1)], T, device="cpu")
+    l, dYs, Xs = group.layers[1], bf16(2, T, M), bf16(2, T, N)
+    V = l.V
+    l.V = gpu(R, N, dtype=torch.float64)
+    for _ in range(2):
+        with pytest.raises(TypeError):
+            group.step(dYs, Xs)
+    l.V = V
+    l.keep_U = False
+    group.step(dYs, Xs)
+    assert calls[-1][1]["V"][1] == V.data_ptr() and calls[-1][1]["U"][1] is None
+    l.W.data = torch.zeros_like(l.W)                 # the same tensor, other memory
+    group.step(dYs, Xs)
+    assert calls[-1][1]["W"][1] == l.W.data_ptr()
