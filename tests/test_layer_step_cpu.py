@@ -235,7 +235,7 @@ def test_a_single_token_has_no_pitch(calls):
 
 
 def test_a_groups_buffers_are_looked_at_again_after_they_were_refused(calls):
-    group = grass.step.GrassLayerGroup([layer(t=1), layer(t=1)], T, device="cpu")
+    group = grass.step.GrassLayerGroup([layer(t=1, K=1 << 30), layer(t=1, K=1 << 30)], T, device="cpu")
     l, dYs, Xs = group.layers[1], bf16(2, T, M), bf16(2, T, N)
     V = l.V
     l.V = gpu(R, N, dtype=torch.float64)
