@@ -67,6 +67,7 @@ struct TcPlan {
   size_t smem_bytes;
   long long ld_part;        // pitch of a split-K partial, elements
   size_t ag_bytes, part_bytes;
+  double us;                // projection_us with its slices taken as equal
 };
 
 // Whether the gathers fetch 64-byte halves of dY's lines instead of whole ones.  A line holds 64
@@ -515,6 +516,8 @@ TcPlan search_plan(int64_t T, int64_t m, int64_t n, int r, bool has_idx, const P
   p.part_bytes = p.split_k > 1
                      ? round_up(static_cast<size_t>(p.split_k) * r * p.ld_part * sizeof(float), 256)
                      : 0;
+  TileChoice equal = {p.gather, p.r_cta, p.r_blocks, p.MB, p.pair, p.split_k, 0, 0};
+  p.us = projection_us(tile_cost(make_problem(T, m, n, r, groups), equal), equal);
   return p;
 }
 
@@ -680,8 +683,9 @@ size_t norm_part_bytes(int64_t m, int64_t n) {
                       sizeof(float), 256);
 }
 
-// Most bytes of partials of a kept gradient, twice L2: 350M gate, 18 slices, 202 MB: 410 us a refresh step
-// against 460 projected again.  A bound on the workspace as much as on the time.
+// Most bytes of partials of a kept gradient, twice L2: a bound on the workspace more than on the time.  Of the
+// timed refreshes 250 have partials of 128 to 256 MB and are kept by the rule below; kept they take 5 %
+// less time than projected again, in the mean (350M gate, 202 MB: 14 %).  Beyond, nothing is gained.
 constexpr double kKeepMostBytes = 256e6;
 
 // fp32 path.  128 x 128 tiles where they can give every SM its two CTAs at 128 tokens or more a
@@ -779,11 +783,15 @@ size_t grad_parts_bytes(int split_k, int64_t m, long long ld) {
 // The plan of a dense gradient that is kept for r selected rows, or false.  Its token slices are those
 // of the projection that it replaces, so that G_C has the same bits: after a state reset the update is the
 // sign of the gradient, and another summation order would turn elements that are zero to rounding.  That makes
-// more partials than the norms alone need; they are written and read once (about 3 TB/s together),
-// which has to cost less than projecting again.
+// more partials than the norms alone need, which has to cost less than projecting again.  The rule sets
+// the two forms' estimates against one another; its factors (the norms' and the update's passes over the
+// partials, their start per slice, the launches saved) are fitted to 13 500 refreshes timed both ways (m, n =
+// 256 .. 5461, T = 256 .. 65536, r = 8 .. 1024).  Over these it costs 0.3 % more than the better form,
+// always keeping 25 %, never 21 %; weighing the partials' bytes alone against the projection cost 0.8 %, and up to
+// 50 % where few rows of a small layer make many slices (T = 13056, 384 x 5461, r = 43: kept 155 us, projected 113).
 bool make_keep_plan(int64_t T, int64_t m, int64_t n, int r, TcPlan* plan) {
   bool small = false;
-  make_norms_plan(T, m, n, &small);
+  const double norms_us = make_norms_plan(T, m, n, &small).us;
   if (!small) return false;
   const TcPlan proj = make_plan(T, m, n, r, true, PlanOpts());
   const int unit = proj.kb_unit * proj.bk;
@@ -797,9 +805,8 @@ bool make_keep_plan(int64_t T, int64_t m, int64_t n, int r, TcPlan* plan) {
   plan->split_k = proj.split_k;
   plan->s_long = proj.s_long;
   for (int z = 0; z <= kTcMaxSlices; ++z) plan->unit_begin[z] = proj.unit_begin[z];
-  const double bytes = static_cast<double>(grad_parts_bytes(plan->split_k, m, plan->ld_part));
-  TileChoice t = {proj.gather, proj.r_cta, proj.r_blocks, proj.MB, proj.pair, proj.split_k, 0, 0};
-  return bytes <= kKeepMostBytes && bytes / 3e6 < projection_us(tile_cost(make_problem(T, m, n, r, 1), t), t) + 6.0;
+  return static_cast<double>(grad_parts_bytes(plan->split_k, m, plan->ld_part)) <= kKeepMostBytes &&
+         1.7 * (plan->us - norms_us) + 0.2 * plan->split_k < proj.us + 9.0;
 }
 
 // The same where the workspace of the norms has room for the partials.
@@ -1219,13 +1226,13 @@ int refresh_projection_refused(const grass_step_t* a, size_t norm_ws_bytes) {
   TcPlan plan;
   if (a->dt == GRASS_F32) {
     const Fp32Plan fp = make_fp32_plan(a->T, a->n, a->r, a->r);
-    return fp.split > 1 && !keeps_fp32(a->T, a->m, a->n, a->r, norm_ws_bytes) &&
-                   (a->ws == nullptr || !aligned_to(a->ws, 256) || a->ws_bytes < fp.part_bytes)
+    return fp.split > 1 && (a->ws == nullptr || !aligned_to(a->ws, 256) || a->ws_bytes < fp.part_bytes) &&
+                   !keeps_fp32(a->T, a->m, a->n, a->r, norm_ws_bytes)
                ? GRASS_ERR_WORKSPACE : GRASS_OK;
   }
-  if (keeps(a->T, a->m, a->n, a->r, norm_ws_bytes, &plan)) return GRASS_OK;
   plan = make_plan(a->T, a->m, a->n, a->r, true, PlanOpts());
-  return plan_refused(plan, a->T, plan_ws_bytes(plan, 1), a->ws, a->ws_bytes);
+  const int refused = plan_refused(plan, a->T, plan_ws_bytes(plan, 1), a->ws, a->ws_bytes);
+  return refused != GRASS_OK && keeps(a->T, a->m, a->n, a->r, norm_ws_bytes, &plan) ? GRASS_OK : refused;
 }
 
 // Row norms of dY^T X; keep (may be NULL) learns where the gradient was formed, if it was.

@@ -177,6 +177,23 @@ def test_a_plan_for_a_new_token_count_costs_little_host_time(lib):
     assert best < 120e-6
 
 
+@pytest.mark.parametrize("T,m,n,r,kept", [
+    # few rows of a small layer: their many token slices make partials that cost more than projecting again
+    # (kept 109 .. 231 us, projected 97 .. 174)
+    (26171, 384, 2444, 11, False), (13056, 384, 5461, 43, False), (62493, 640, 1376, 62, False),
+    (57414, 512, 1376, 24, False), (2304, 768, 263, 8, False), (47616, 3072, 256, 166, False),
+    # 350M gate and q, 60M q and down, a short batch: kept 14 to 40 % faster
+    (65536, 2736, 1024, 256, True), (65536, 1024, 1024, 256, True), (65536, 512, 512, 128, True),
+    (65536, 512, 1376, 128, True), (2048, 512, 512, 64, True),
+    (65536, 11008, 4096, 1024, False),               # large: never formed
+])
+def test_a_gradient_is_kept_where_that_was_measured_faster(lib, T, m, n, r, kept):
+    assert binding.grass_refresh_keeps_gradient(T, m, n, r, binding.BF16) == kept
+    # no workspace for partials that are not kept
+    norms = binding.grass_grad_row_norms_workspace_bytes(T, m, n, binding.BF16)
+    assert (binding.grass_refresh_workspace_bytes(T, m, n, r, binding.BF16) > norms) == kept
+
+
 def test_workspace_queries_are_host_only_and_monotone(lib):
     assert binding.grass_select_workspace_bytes(4096, 256, binding.SEL_TOPR) >= 256
     a = binding.grass_select_workspace_bytes(4096, 256, binding.SEL_MULTINOMIAL_NORM)
