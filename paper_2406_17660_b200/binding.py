@@ -483,7 +483,10 @@ class LayerStepCall:
         self.args = a = LayerStep()
         self._ref = ctypes.byref(a)
         self._slots = (a.dY, a.X, a.idx, a.rho, a.Gc, a.M, a.V, a.U, a.W)
-        self._launch = load_library().grass_layer_step
+        self._refresh = f = Refresh()
+        self._refresh_ref = ctypes.byref(f)
+        lib = load_library()
+        self._launch, self._launch_refresh = lib.grass_layer_step, lib.grass_refresh_step
         self._now = self._held = self._pointers = None
 
     def __reduce__(self):
@@ -581,15 +584,17 @@ class LayerStepCall:
                 norms, norm_ws, select_ws) -> None:
         """grass_refresh_step on layer 0."""
         self._scalars(1, ws, (lr, beta1, beta2, eps, alpha), step)
-        a = self.args
-        _require(norms, torch.float32, "norms")
-        if norms.numel() < a.m:
+        if norms.dtype is not torch.float32 or not norms.is_cuda:
+            raise TypeError("norms must be a CUDA tensor of torch.float32")
+        if norms.numel() < self.args.m:
             raise ValueError("norms must hold one value per row")
-        f = Refresh(method, layer_id, epoch, 1 if reset_state else 0, seed, norms.data_ptr(),
-                    norm_ws.data_ptr(), norm_ws.numel() * norm_ws.element_size(), None, 0)
-        if select_ws is not None:
-            f.select_ws, f.select_ws_bytes = select_ws.data_ptr(), select_ws.numel() * select_ws.element_size()
-        _check(load_library().grass_refresh_step(self._ref, ctypes.byref(f), _stream()), "grass_refresh_step")
+        f = self._refresh
+        f.method, f.layer_id, f.epoch, f.reset_state, f.seed = method, layer_id, epoch, 1 if reset_state else 0, seed
+        f.norms, f.norm_ws, f.norm_ws_bytes = norms.data_ptr(), norm_ws.data_ptr(), norm_ws.nbytes
+        f.select_ws, f.select_ws_bytes = (None, 0) if select_ws is None else (select_ws.data_ptr(), select_ws.nbytes)
+        status = self._launch_refresh(self._ref, self._refresh_ref, _stream())
+        if status != 0:
+            raise GrassError(status, "grass_refresh_step")
 
 
 def grass_layer_step(dYs, Xs, idxs, rhos, Gcs, Ms, Vs, Us, Ws, ws, lr, beta1, beta2, eps, step,

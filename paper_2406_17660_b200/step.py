@@ -86,21 +86,17 @@ class GrassLayer:
         """Whether a program has put its own in the place of refresh(): then it is that which is called."""
         return type(self).refresh is not GrassLayer.refresh or "refresh" in self.__dict__
 
-    def _marshal(self, dY, X):
-        """The layer's call with its buffers and these inputs filled in."""
-        if self._call is None:
-            self._call = B.LayerStepCall()
-        self._call.state(0, self.idx, self.rho, self.Gc, self.M, self.V, self.U if self.keep_U else None,
-                         self.W, self.side == "cols")
-        self._call.inputs(0, dY, X)
-        return self._call
-
     def _refresh_step(self, dY, X, of, step):
         """A refresh iteration in one call, with the hyper-parameters of layer `of`."""
-        ws = self.ws
-        self._marshal(dY, X).refresh(ws.project_ws, of.lr, of.beta1, of.beta2, of.eps, step, of.alpha,
-                                     self.method, self.seed, self.layer_id, self.t // self.K,
-                                     self.reset_state, ws.norms, ws.norm_ws, ws.select_ws)
+        ws, call = self.ws, self._call
+        if call is None:
+            call = self._call = B.LayerStepCall()
+        call.state(0, self.idx, self.rho, self.Gc, self.M, self.V, self.U if self.keep_U else None,
+                   self.W, self.side == "cols")
+        call.inputs(0, dY, X)
+        call.refresh(ws.project_ws, of.lr, of.beta1, of.beta2, of.eps, step, of.alpha,
+                     self.method, self.seed, self.layer_id, self.t // self.K,
+                     self.reset_state, ws.norms, ws.norm_ws, ws.select_ws)
 
     def step(self, dY, X):
         """One iteration of Algorithm 1 for this layer; dY (T x m), X (T x n) on the device."""
@@ -113,8 +109,14 @@ class GrassLayer:
                     self.adam_step = 0
                 self._refresh_step(dY, X, self, self.adam_step + 1)
             else:
-                self._marshal(dY, X).launch(1, self.ws.project_ws, self.lr, self.beta1, self.beta2, self.eps,
-                                            self.adam_step + 1, self.alpha)
+                call = self._call
+                if call is None:
+                    call = self._call = B.LayerStepCall()
+                call.state(0, self.idx, self.rho, self.Gc, self.M, self.V, self.U if self.keep_U else None,
+                           self.W, self.side == "cols")
+                call.inputs(0, dY, X)
+                call.launch(1, self.ws.project_ws, self.lr, self.beta1, self.beta2, self.eps,
+                            self.adam_step + 1, self.alpha)
             self.adam_step += 1
             self.t += 1
             return
