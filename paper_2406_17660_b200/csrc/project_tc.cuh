@@ -651,31 +651,38 @@ project_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
           break;
         }
         uint8_t* stage = tiles + s * STAGE_BYTES + X_SLABS * kTcSlabBytes;
+        // 32 loads a lane in flight (all tokens of this warp's share, or half of them where the CTA
+        // stages two slabs: with all of both, 384 bytes of spills; 512 x 256 x 4, T = 65536, r = 128: 150 us,
+        // 101 so), then the stores: the gather is latency-bound otherwise.  The loads are
+        // unconditional (clamped, the value discarded at the store): under a per-lane condition
+        // the warp would wait for each before issuing the next.
+        constexpr int NT = kTcBK / GW, FLIGHT = NT / A_SLABS;
 #pragma unroll
-        for (int a = 0; a < A_SLABS; ++a) {
-          // all loads of this warp's share of the slab first (kTcBK / GW tokens x 2 per lane in
-          // flight), then the stores: the gather is latency-bound otherwise.  The loads are
-          // unconditional (clamped, the value discarded at the store): under a per-lane condition
-          // the warp would wait for each before issuing the next.
-          constexpr int NT = kTcBK / GW;
-          unsigned short v0[NT], v1[NT];
+        for (int k0 = 0; k0 < NT; k0 += FLIGHT) {
+          unsigned short v[FLIGHT][A_SLABS][2];
 #pragma unroll
-          for (int k = 0; k < NT; ++k) {
-            const int tok = tok0 + g + k * GW;
+          for (int k = 0; k < FLIGHT; ++k) {
+            const int tok = tok0 + g + (k0 + k) * GW;
             const unsigned short* line = src + static_cast<long long>(tok < p.T ? tok : p.T - 1) * p.lddy;
-            v0[k] = ptx::ld_nc_u16(line + max(rows[a][0], 0));
-            v1[k] = ptx::ld_nc_u16(line + max(rows[a][1], 0));
+#pragma unroll
+            for (int a = 0; a < A_SLABS; ++a) {
+              v[k][a][0] = ptx::ld_nc_u16(line + max(rows[a][0], 0));
+              v[k][a][1] = ptx::ld_nc_u16(line + max(rows[a][1], 0));
+            }
           }
 #pragma unroll
-          for (int k = 0; k < NT; ++k) {
-            const int tt = g + k * GW;
-            uint8_t* rowp = stage + a * kTcSlabBytes + tt * 128;
+          for (int k = 0; k < FLIGHT; ++k) {
+            const int tt = g + (k0 + k) * GW;
             const int sw = tt & 7;
             const bool live = tok0 + tt < p.T;
-            *reinterpret_cast<unsigned short*>(rowp + (((lane >> 3) ^ sw) << 4) + (lane & 7) * 2) =
-                live && rows[a][0] >= 0 ? v0[k] : 0;
-            *reinterpret_cast<unsigned short*>(rowp + ((((lane >> 3) + 4) ^ sw) << 4) + (lane & 7) * 2) =
-                live && rows[a][1] >= 0 ? v1[k] : 0;
+#pragma unroll
+            for (int a = 0; a < A_SLABS; ++a) {
+              uint8_t* rowp = stage + a * kTcSlabBytes + tt * 128;
+              *reinterpret_cast<unsigned short*>(rowp + (((lane >> 3) ^ sw) << 4) + (lane & 7) * 2) =
+                  live && rows[a][0] >= 0 ? v[k][a][0] : 0;
+              *reinterpret_cast<unsigned short*>(rowp + ((((lane >> 3) + 4) ^ sw) << 4) + (lane & 7) * 2) =
+                  live && rows[a][1] >= 0 ? v[k][a][1] : 0;
+            }
           }
         }
         ptx::fence_proxy_async_smem();   // generic writes -> visible to the MMA's async proxy
