@@ -181,8 +181,11 @@ TileCost tile_cost(const Problem& q, const TileChoice& t) {
   k.c *= unit / 32.0;
   k.f = 0.42 + (t.pair ? 2.0 : 0.0) + 4.5 * t.mb * t.r_cta / 512;
   // row-norm epilogue, few tokens: with two accumulator sets the drain of one tile hides behind the
-  // MMAs of the next (stores do not: they meet the next tile's loads in L2)
-  k.drain = t.gather == 0 && T <= 1536 && t.mb * t.r_cta <= 256 ? 4.5 * t.mb * t.r_cta / 512 : 0;
+  // MMAs of the next (stores do not: they meet the next tile's loads in L2).  Not where a pair's tile has
+  // 128 columns: its MMAs are too short to hide a pair's start as well (70 shapes: 8 % slower than tiles as
+  // large as TMEM allows, where the model had them 20 % faster)
+  const int columns = t.mb * t.r_cta;
+  k.drain = t.gather == 0 && T <= 1536 && columns <= 256 && !(t.pair && columns <= 128) ? 4.5 * columns / 512 : 0;
   const double dy_mb = groups * 2.0 * T * m * q.lines * MBYTE, x_mb = groups * 2.0 * T * n * MBYTE;
   const double ag_mb = groups * 2.0 * T * t.r_cta * t.r_blocks * MBYTE, out_mb = groups * 4.0 * r * n * MBYTE;
   // load-unit time of one pass over the picks, and how many lines a load instruction of 32 spans
