@@ -834,6 +834,15 @@ int plan_refused(const TcPlan& plan, int64_t T, size_t need, const void* ws, siz
   return GRASS_OK;
 }
 
+// Rows of up to 128, 256 and 512 columns (four a thread) share a CTA.
+cudaError_t launch_row_norms(const float* part, long long ld, long long stride, int split_k, int64_t m, int64_t n,
+                             float* norms, cudaStream_t s) {
+  const int threads = n <= 128 ? 32 : n <= 256 ? 64 : n <= 512 ? 128 : 256, rows = 256 / threads;
+  auto kernel = threads < 256 ? splitk_rownorms_kernel<true> : splitk_rownorms_kernel<false>;
+  return launch_kernel(kernel, static_cast<unsigned>((m + rows - 1) / rows), 256, 0, s, true, part, ld, stride,
+                       split_k, static_cast<int>(m), static_cast<int>(n), threads, norms);
+}
+
 // Projection of `count` same-shaped layers in one set of launches (count = 1 for the plain
 // call).  norms != NULL (count must be 1): row-norm mode (idx NULL, r == m): the GEMM's epilogue
 // reduces squares instead of storing the gradient, then the partial sums are finalised.
@@ -981,9 +990,7 @@ int project_bf16(int count, const void* const* dY, int64_t lddy, const void* con
                                    true, p.norm_part, p.ld_norm, static_cast<int>((n + 31) / 32),
                                    static_cast<int>(m), norms));
     else
-      GRASS_CUDA_TRY(launch_kernel(splitk_rownorms_kernel, static_cast<unsigned>(m), 256, 0, s, true,
-                                   part[0], plan.ld_part, p.split_stride, plan.split_k,
-                                   static_cast<int>(m), static_cast<int>(n), norms));
+      GRASS_CUDA_TRY(launch_row_norms(part[0], plan.ld_part, p.split_stride, plan.split_k, m, n, norms, s));
     if (stored) *keep = {keep->r, part[0], plan.ld_part, p.split_stride, plan.split_k};
     return GRASS_OK;
   }
@@ -1087,8 +1094,7 @@ int project_fp32(const void* dY, int64_t lddy, const void* X, int64_t ldx, int64
     // row-norm mode (idx NULL, r == m): the norms straight from the partials
     ProfileScope prof(GRASS_K_ROW_NORMS, s);
     const long long stride = static_cast<long long>(r) * fp.ld_part;
-    GRASS_CUDA_TRY(launch_kernel(splitk_rownorms_kernel, static_cast<unsigned>(m), 256, 0, s, true, out,
-                                 ld_out, stride, fp.split, r, static_cast<int>(n), norms));
+    GRASS_CUDA_TRY(launch_row_norms(out, ld_out, stride, fp.split, m, n, norms, s));
     if (keep != nullptr) *keep = {keep->r, out, static_cast<long long>(ld_out), stride, fp.split};
     return GRASS_OK;
   }

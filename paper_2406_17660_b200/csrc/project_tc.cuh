@@ -900,20 +900,26 @@ splitk_reduce_kernel(const ReduceGroup grp, long long ld_part, long long split_s
 }
 
 // Row norms from split-K partials of a small dense gradient: norms[j] = sqrt(sum_c (sum_s
-// part[s][j][c])^2).  One CTA per row; splits added in increasing s, four columns a thread and
-// four splits in flight (the partials' pitch is a multiple of four and their base aligned; the
+// part[s][j][c])^2).  A CTA takes 256 / row_threads rows; splits added in increasing s, four columns a thread
+// and four splits in flight (the partials' pitch is a multiple of four and their base aligned; the
 // columns past n of the last four are masked out), columns in a fixed thread-strided order, then
-// a shuffle tree and one shared-memory hop: bit-reproducible.
+// a shuffle tree and one shared-memory hop: bit-reproducible, whatever row_threads is.
+// Bound by the latency of its loads where rows are short, so no thread is left without any (5461 rows of 91
+// columns in 13 splits: 37 us with a CTA per row).
+// SHORT: row_threads as given (32, 64 or 128); else 256, known to the compiler.
+template <bool SHORT>
 __global__ void __launch_bounds__(256)
 splitk_rownorms_kernel(const float* part, long long ld_part, long long split_stride,
-                       int split_k, int m, int n, float* norms) {
+                       int split_k, int m, int n, int short_row_threads, float* norms) {
   __shared__ float s_part[8];
   grid_dep_launch();
   grid_dep_wait();
-  const int j = blockIdx.x;
+  const int row_threads = SHORT ? short_row_threads : 256;
+  const int warp = threadIdx.x >> 5, t = threadIdx.x & (row_threads - 1);
+  const int j = blockIdx.x * (256 / row_threads) + threadIdx.x / row_threads;
   const float* row = part + static_cast<long long>(j) * ld_part;
   float acc = 0.f;
-  for (int c = 4 * threadIdx.x; c < n; c += 4 * 256) {
+  for (int c = j < m ? 4 * t : n; c < n; c += 4 * row_threads) {
     const float* p = row + c;
     float4 g = *reinterpret_cast<const float4*>(p);
     for (int s = 1; s < split_k; s += 4) {
@@ -934,12 +940,12 @@ splitk_rownorms_kernel(const float* part, long long ld_part, long long split_str
     if (c + 3 < n) acc = fmaf(g.w, g.w, acc);
   }
   acc = warp_sum(acc);
-  if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = acc;
+  if ((threadIdx.x & 31) == 0) s_part[warp] = acc;
   __syncthreads();
-  if (threadIdx.x < 32) {
-    float v = threadIdx.x < 8 ? s_part[threadIdx.x] : 0.f;
+  if (t < 32) {                          // the row's first warp adds up its warps' sums
+    float v = t < row_threads / 32 ? s_part[warp + t] : 0.f;
     v = warp_sum(v);
-    if (threadIdx.x == 0) norms[j] = sqrtf(v);
+    if (t == 0 && j < m) norms[j] = sqrtf(v);
   }
 }
 

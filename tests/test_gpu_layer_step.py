@@ -94,3 +94,22 @@ def test_the_column_form_rounds_as_the_column_scatter(dtype, lengths):
     grass.grass_device_status()
     for name, want in (("M", M), ("V", V), ("U", U), ("W", W)):
         assert torch.equal(getattr(l, name), want), name
+
+
+@pytest.mark.parametrize("m,n", [(37, 4), (300, 91), (65, 128), (129, 129), (700, 203), (50, 256), (33, 257), (90, 512),
+                                 (21, 513), (40, 1030)])
+@pytest.mark.parametrize("dtype", [BF16, torch.float32], ids=["bf16", "fp32"])
+def test_norms_of_short_rows(m, n, dtype):
+    """Row norms from split partials, at the row lengths where the number of rows a CTA takes changes; the rows
+    past the last do not reach the norms."""
+    T = 4096
+    dY, X, _ = inputs(T, m, n, seed=5, dtype=dtype)
+    code = grass.BF16 if dtype == BF16 else grass.F32
+    ws = torch.full((grass.grass_grad_row_norms_workspace_bytes(T, m, n, code),), 0x7F, dtype=torch.uint8, device=DEV)
+    norms = torch.full((m + 64,), -1.0, device=DEV)
+    grass.grass_grad_row_norms(dY, X, norms[:m], ws)
+    grass.grass_device_status()
+    want = (dY.double().T @ X.double()).norm(dim=1)
+    # exact products, fp32 sums over 4096 tokens in slices and n columns
+    assert float(((norms[:m].double() - want).abs() / want).max()) <= 1e-5
+    assert bool((norms[m:] == -1).all())
