@@ -225,3 +225,51 @@ def test_update_kernels_stay_inside_their_buffers(m, n, ld, r, wdtype):
         grass.grass_scatter_update_cols(Wc.t, Uc, cidx, rho, 0.25)
         grass.grass_device_status()
         Wc.check("W (column form)")
+
+
+STEP_SHAPES = [
+    # T, m, n, r
+    (777, 700, 1001, 100),             # rows of an odd length, split tokens
+    (31, 64, 64, 64),                  # fewer tokens than a block, every row selected
+    (640, 2048, 3000, 1000),           # large update, unsplit
+    (300, 4096, 640, 33),
+    (2500, 256, 256, 64),              # gathered inside the GEMM
+]
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32], ids=["bf16", "fp32"])
+@pytest.mark.parametrize("side", ["rows", "cols"])
+@pytest.mark.parametrize("T,m,n,r", STEP_SHAPES)
+def test_layer_and_refresh_steps_stay_inside_their_buffers(T, m, n, r, side, dtype):
+    """grass_layer_step and grass_refresh_step (with room to keep the gradient, and without): every buffer that
+    they write, workspaces of exactly the stated size, and the layer's padding."""
+    dt = grass.BF16 if dtype == torch.bfloat16 else grass.F32
+    rng = np.random.default_rng(T + r)
+    a, b = (syn._padded(f(T, k, dtype, seed0=1).to(DEV), syn.pad_to(k, 8)) for f, k in ((syn.make_dY, m), (syn.make_X, n)))
+    rows, cols = (m, n) if side == "rows" else (n, m)
+    method = grass.SEL_MULTINOMIAL_NORM
+    norm_bytes = (grass.grass_refresh_workspace_bytes(T, m, n, r, dt), grass.grass_grad_row_norms_workspace_bytes(T, m, n, dt))
+    for norm_ws_bytes in (None, *norm_bytes):
+        W = Guarded(rows, cols, dtype, ld=syn.pad_to(cols, 8) + 8, init=torch.randn((rows, cols), device=DEV).to(dtype))
+        idx, rho = Guarded(1, r, torch.int32), Guarded(1, r, torch.float32)
+        idx.vec().copy_(_idx(m, r, rng, dup=r < m)); rho.vec().fill_(1.0)
+        M, V = (Guarded(r, n, torch.float32, ld=n + 3, init=torch.rand((r, n), device=DEV)) for _ in range(2))
+        U, Gc = Guarded(r, n, torch.float32, ld=n + 3), Guarded(r, n, torch.float32, ld=n + 5)
+        ws = workspace(grass.grass_project_workspace_bytes(T, m, n, r, dt))
+        call = grass.binding.LayerStepCall()
+        call.state(0, idx.vec(), rho.vec(), Gc.t, M.t, V.t, U.t, W.t, side == "cols")
+        call.inputs(0, a, b)
+        hyper = (1e-3, 0.9, 0.999, 1e-8, 3, 0.25)
+        written = dict(W=W, idx=idx, rho=rho, M=M, V=V, U=U, Gc=Gc, ws=ws)
+        if norm_ws_bytes is None:
+            call.launch(1, ws.vec(), *hyper)
+        else:
+            norms, norm_ws = Guarded(1, m, torch.float32), workspace(norm_ws_bytes)
+            select_ws = workspace(grass.grass_select_workspace_bytes(m, r, method))
+            call.refresh(ws.vec(), *hyper, method, 5, 1, 2, False, norms.vec(), norm_ws.vec(), select_ws.vec())
+            written.update(norms=norms, norm_ws=norm_ws, select_ws=select_ws)
+        grass.grass_device_status()
+        for name, g in written.items():
+            g.check(name)
+        for g in (M, V, U, Gc, W):
+            assert bool(torch.isfinite(g.t.float()).all())

@@ -113,3 +113,161 @@ def test_norms_of_short_rows(m, n, dtype):
     # exact products, fp32 sums over 4096 tokens in slices and n columns
     assert float(((norms[:m].double() - want).abs() / want).max()) <= 1e-5
     assert bool((norms[m:] == -1).all())
+
+
+@pytest.mark.parametrize("r,n", [(585, 1024), (586, 1024), (146, 4096), (147, 4096), (109, 5461), (110, 5461)])
+@pytest.mark.parametrize("repeats", [False, True])
+def test_update_forms_around_their_limits(r, n, repeats):
+    """Elements just below and above where the update changes its kernel: the bits of Adam and the row scatter."""
+    rng = np.random.default_rng(r + n)
+    m = 2 * r
+    idx = torch.tensor(np.sort(rng.choice(m, r, replace=False) if not repeats else (rng.pareto(1.0, r) * 8).astype(int) % m),
+                       dtype=torch.int32, device=DEV)
+    rho, Gc = torch.rand(r, device=DEV) + 0.5, torch.randn((r, n), device=DEV)
+    M, V, W = torch.randn((r, n), device=DEV), torch.rand((r, n), device=DEV), torch.randn((m, n), device=DEV).to(BF16)
+    want = [t.clone() for t in (M, V, W)]
+    U, hp = torch.empty_like(M), (1e-3, 0.9, 0.999, 1e-8, 3)
+    grass.grass_subspace_adam(Gc, want[0], want[1], U, *hp)
+    grass.grass_scatter_update(want[2], U, idx, rho, 0.25)
+    grass.grass_adam_scatter(Gc, M, V, None, W, idx, rho, *hp, 0.25)
+    grass.grass_device_status()
+    for got, w in zip((M, V, W), want):
+        assert torch.equal(got, w)
+
+
+def layers_of(count, T, m, n, r, K=1 << 30, t=1, reset=True, seed=0):
+    """`count` layers of one shape in mid-epoch, and their inputs."""
+    ws = grass.step.GrassWorkspace([(m, n)], T, r, BF16, grass.SEL_TOPR)
+    layers, dYs, Xs = [], [], []
+    for g in range(count):
+        dY, X, W = inputs(T, m, n, seed=seed, proj=g)
+        l = grass.GrassLayer(W, r, grass.SEL_TOPR, K, 0.25, 1e-3, reset_state=reset, seed=3, layer_id=g, workspace=ws)
+        l.idx.copy_(rows_of(m, r, g))
+        l.rho.copy_(torch.rand(r, generator=torch.Generator().manual_seed(g)) + 0.5)
+        l.M.normal_(); l.V.uniform_(0.5, 1.5)
+        l.t, l.adam_step = t, 6
+        layers.append(l); dYs.append(dY); Xs.append(X)
+    return layers, dYs, Xs
+
+
+def state_of(layers):
+    return [[getattr(l, k).clone() for k in ("M", "V", "U", "W")] for l in layers]
+
+
+def check_update(layers, before, step):
+    """M, V, U and W are those of the separate update from the layers' own G_C, bit for bit."""
+    for l, (M, V, U, W) in zip(layers, before):
+        grass.grass_adam_scatter(l.Gc, M, V, U, W, l.idx, l.rho, l.lr, l.beta1, l.beta2, l.eps, step, l.alpha)
+        for k, want in (("M", M), ("V", V), ("U", U), ("W", W)):
+            assert torch.equal(getattr(l, k), want), k
+
+
+MODES = [
+    # layers, T, m, n, r, and what the step's own plan picks: gather, pair, short slices
+    (1, 1000, 256, 256, 100, grass.GATHER_PREPASS, 0, False),
+    (1, 3000, 1024, 2048, 1024, grass.GATHER_PREPASS, 1, False),
+    (2, 9000, 1024, 5461, 1024, grass.GATHER_PREPASS, 1, True),
+    (1, 1000, 256, 256, 64, grass.GATHER_IN_CTA, 0, True),
+    (4, 3000, 256, 256, 256, grass.GATHER_IN_CTA, 1, True),
+    (1, 6000, 4096, 5461, 1024, grass.GATHER_COOPERATIVE, 1, False),
+    (1, 9000, 4096, 5461, 512, grass.GATHER_COOPERATIVE, 1, False),
+]
+
+
+@pytest.mark.parametrize("count,T,m,n,r,gather,pair,short", MODES)
+def test_every_gather_hands_over_to_the_update(count, T, m, n, r, gather, pair, short):
+    """Each gather, single CTAs and pairs, long and short slices, followed by the update in one call, eagerly and
+    from a CUDA graph: G_C of the projection calls to summation order, the update's bits."""
+    p = grass.grass_step_plan(count, T, m, n, r)
+    assert (p["gather"], p["cta_pair"], p["short_slices"] > 0) == (gather, pair, short)
+    layers, dYs, Xs = layers_of(count, T, m, n, r)
+    stepper = layers[0] if count == 1 else grass.step.GrassLayerGroup(layers, T)
+    args = (dYs[0], Xs[0]) if count == 1 else (dYs, Xs)
+    before = state_of(layers)
+    stepper.step(*args)
+    grass.grass_device_status()
+    full = torch.empty(grass.grass_project_batched_workspace_bytes(count, T, m, n, r), dtype=torch.uint8, device=DEV)
+    want = [torch.empty_like(l.Gc) for l in layers]
+    grass.grass_project_grad_batched(dYs, Xs, [l.idx for l in layers], [l.rho for l in layers], r, want, full)
+    for l, w in zip(layers, want):
+        assert rel(l.Gc, w) <= 1e-5
+    check_update(layers, before, 7)
+    eager = [l.Gc.clone() for l in layers]
+    before = state_of(layers)
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        stepper.step(*args)
+    graph.replay()
+    grass.grass_device_status()
+    for l, g in zip(layers, eager):
+        assert torch.equal(l.Gc, g)
+    check_update(layers, before, 8)
+
+
+@pytest.mark.parametrize("reset", [True, False])
+@pytest.mark.parametrize("T,m,n,r,kept", [(4096, 512, 520, 100, True), (256, 4096, 4100, 200, False)])
+def test_a_group_against_its_layers_stepped_singly(T, m, n, r, kept, reset):
+    """A refresh that keeps its gradient has the bits of the layers' own; one that does not, those of the batched
+    projection; then a regular step."""
+    assert grass.grass_refresh_keeps_gradient(T, m, n, r, grass.BF16) == kept
+    (grouped, dYs, Xs), (single, _, _) = (layers_of(3, T, m, n, r, K=4, t=4, reset=reset) for _ in range(2))
+    for a, b in zip(grouped, single):
+        b.M.copy_(a.M); b.V.copy_(a.V)
+    before = state_of(grouped)
+    group = grass.step.GrassLayerGroup(grouped, T)
+    group.step(dYs, Xs)
+    for l, dY, X in zip(single, dYs, Xs):
+        l.step(dY, X)
+    grass.grass_device_status()
+    for a, b in zip(grouped, single):
+        assert torch.equal(a.idx, b.idx) and torch.equal(a.rho, b.rho)
+        assert (a.t, a.adam_step) == (b.t, b.adam_step) == (5, 1 if reset else 7)
+        assert rel(a.Gc, b.Gc) <= 1e-5
+        if kept:
+            for k in ("Gc", "M", "V", "U", "W"):
+                assert torch.equal(getattr(a, k), getattr(b, k)), k
+    if not kept:
+        want = [torch.empty_like(l.Gc) for l in grouped]
+        grass.grass_project_grad_batched(dYs, Xs, [l.idx for l in grouped], [l.rho for l in grouped], r, want, group.ws)
+        for l, w in zip(grouped, want):
+            assert torch.equal(l.Gc, w)
+    if reset:
+        for b in before:
+            b[0].zero_(); b[1].zero_()
+    check_update(grouped, before, 1 if reset else 7)
+    before = state_of(grouped)
+    group.step(dYs, Xs)
+    check_update(grouped, before, 2 if reset else 8)
+
+
+@pytest.mark.parametrize("count,T,m,n,r", [
+    (4, 32768, 4096, 4096, 1024), (2, 32768, 11008, 4096, 256),     # 7B q,k,v,o and gate,up
+    (1, 65536, 2048, 5461, 512), (2, 65536, 5461, 2048, 64),        # 1B down and gate,up
+    (1, 65536, 1024, 2736, 256), (4, 65536, 512, 512, 128),         # 350M down, 60M q,k,v,o
+    (1, 4096, 5120, 13824, 1024),                                   # 13B down, one micro-batch
+])
+def test_regular_steps_at_full_size(count, T, m, n, r):
+    """The tiling that regular steps run at the LLaMA shapes, on sampled rows in 64 bits, and its update."""
+    ws = grass.step.GrassWorkspace([(m, n)], T, r, BF16, grass.SEL_TOPR)
+    layers, dYs, Xs = [], [], []
+    gen = torch.Generator(device=DEV).manual_seed(T + m)
+    for g in range(count):
+        dY, X = (torch.empty((T, syn.pad_to(k, 8)), dtype=BF16, device=DEV).normal_(generator=gen)[:, :k] for k in (m, n))
+        W = torch.empty((m, syn.pad_to(n, 8)), dtype=BF16, device=DEV).normal_(generator=gen)[:, :n]
+        l = grass.GrassLayer(W, r, grass.SEL_TOPR, 1 << 30, 0.25, 1e-3, layer_id=g, workspace=ws)
+        l.idx.copy_(rows_of(m, r, g)); l.t = 1
+        l.V.fill_(1.0)
+        layers.append(l); dYs.append(dY); Xs.append(X)
+    before = state_of(layers)
+    if count == 1:
+        layers[0].step(dYs[0], Xs[0])
+    else:
+        grass.step.GrassLayerGroup(layers, T).step(dYs, Xs)
+    grass.grass_device_status()
+    for l, dY, X in zip(layers, dYs, Xs):
+        js = torch.randint(r, (4,), device=DEV, generator=gen)
+        want = sum(dY[t:t + 8192][:, l.idx[js].long()].double().T @ X[t:t + 8192].double() for t in range(0, T, 8192))
+        assert rel(l.Gc[js], want) <= 1e-4
+        assert float((l.Gc[js] - want).abs().max() / want.abs().max()) <= 1e-4
+    check_update(layers, before, 1)
