@@ -225,6 +225,12 @@ def run_reference(args):
 
 
 # ----------------------------------------------------------------------------- GPU arm
+def dy_touched_share(m, r):
+    """Share of dY that gathering r of m columns fetches: 128-byte lines (64 columns) that hold a pick, or
+    their 64-byte halves where picks are sparse (the library's rule: r/m < 1/10)."""
+    return 1.0 - (1.0 - r / m) ** (32 if 10 * r < m else 64)
+
+
 def aggregate_max(local_ms: float, dist_mod=None) -> float:
     """Max over ranks of a duration (the slowest replica bounds the job)."""
     if dist_mod is None or not dist_mod.is_initialized():
@@ -400,11 +406,11 @@ def measure_workload(ctx, name, r, steps, warmup, want_e2e, want_cpu, args):
                       if k in per_kernel)
         # algorithmic bytes of the projection per layer-step: X once, the r selected columns of
         # dY once, G_C out (2Tn + 2Tr + 4rn); per refresh: X and dY once (2Tn + 2Tm).  What the
-        # memory system cannot avoid touching is larger: every 128-byte line of dY that holds a
-        # selected column (measured with ncu), i.e. 2Tm (1 - (1 - r/m)^64) instead of 2Tr.
+        # memory system cannot avoid touching is larger: every part of a line of dY that is fetched
+        # and holds a selected column (dy_touched_share) instead of 2Tr.
         rs = [(min(wl.r, m), m, n) for _, m, n in wl.shapes]
         alg_reg = sum(2.0 * wl.T * n + 2.0 * wl.T * r_ + 4.0 * r_ * n for r_, m, n in rs) * wl.layers
-        touched_reg = sum(2.0 * wl.T * n + 2.0 * wl.T * m * (1.0 - (1.0 - r_ / m) ** 64) + 4.0 * r_ * n
+        touched_reg = sum(2.0 * wl.T * n + 2.0 * wl.T * m * dy_touched_share(m, r_) + 4.0 * r_ * n
                           for r_, m, n in rs) * wl.layers
         dense = sum(2.0 * wl.T * n + 2.0 * wl.T * m for r_, m, n in rs) * wl.layers
         # the launches of the regular steps only: the dense GEMMs of refresh iterations are the
@@ -434,7 +440,8 @@ def measure_workload(ctx, name, r, steps, warmup, want_e2e, want_cpu, args):
                     "frac_of_burst_peak": tensor_side["achieved"] / burst,
                     "frac_of_sustained_peak": tensor_side["achieved"] / sustained,
                     # the projection as the method sees it: selected-column gather (inside the GEMM
-                    # kernel unless a pre-pass is used) + GEMM + split-K reduce, same flops
+                    # kernel unless a pre-pass is used) + GEMM + split-K reduce, same flops (a regular
+                    # step's reduce is part of its update: see hbm.adam_scatter)
                     "path": {"kernels": [k for k in ("gather", "project_tc", "splitk_reduce")
                                          if k in per_kernel],
                              "ms": path_ms, "achieved": flops_proj / (path_ms * 1e-3) / 1e12,
@@ -456,6 +463,9 @@ def measure_workload(ctx, name, r, steps, warmup, want_e2e, want_cpu, args):
                     "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                     "peak_source": "148 SMs x 128 fp32 lanes x 2 flop x 1.965 GHz", "traffic": None}
     hbm = {}
+    # what a regular step of every unit does (the fp32 path has no such plan)
+    plans = [grass.grass_step_plan(len(u["layers"]), wl.T, u["layers"][0].m, u["layers"][0].n, u["layers"][0].r)
+             if wl.dtype == torch.bfloat16 else {"token_slices": 1, "gather": 0} for u in units]
     if regular_steps or refresh_steps:
         rn = sum(min(wl.r, m) * n for _, m, n in wl.shapes) * wl.layers
         wbytes = 2 if wl.dtype == torch.bfloat16 else 4
@@ -466,14 +476,23 @@ def measure_workload(ctx, name, r, steps, warmup, want_e2e, want_cpu, args):
             b = (4.0 + 2 * wbytes) * rn * steps
             hbm["scatter"] = {"gbs": b / (per_kernel["scatter"]["ms"] * 1e-3) / 1e9}
         if "adam_scatter" in per_kernel:
-            b = (20.0 + 2 * wbytes) * rn * steps      # g, M, V in; M, V out; W in and out
+            # M, V in and out, W in and out, and the gradient: read, or summed from the partials of the
+            # step's token slices and written (on refreshes taken as read)
+            b = (20.0 + 2 * wbytes) * rn * steps
+            for unit, plan in zip(units, plans):
+                if plan["token_slices"] > 1:
+                    l = unit["layers"][0]
+                    b += 4.0 * plan["token_slices"] * l.r * l.n * len(unit["layers"]) * len(regular_steps)
             hbm["adam_scatter"] = {"gbs": b / (per_kernel["adam_scatter"]["ms"] * 1e-3) / 1e9}
         if "gather" in per_kernel:
-            # a pre-pass (only when asked for): algorithmic bytes 2Tr in + 2Tr out per layer; what
-            # it must touch is every 128-byte line of dY that holds a selected column, and the copy
-            alg = sum(4.0 * wl.T * min(wl.r, m) for _, m, n in wl.shapes) * wl.layers * steps
-            touched = sum(2.0 * wl.T * m * (1.0 - (1.0 - min(wl.r, m) / m) ** 64) +
-                          2.0 * wl.T * min(wl.r, m) for _, m, n in wl.shapes) * wl.layers * steps
+            # the separate gather, of the units whose regular step has one: algorithmic bytes 2Tr in + 2Tr
+            # out per layer; what it must touch is dY's share and the copy
+            alg = touched = 0.0
+            for unit, plan in zip(units, plans):
+                l, k = unit["layers"][0], len(unit["layers"]) * len(regular_steps)
+                if plan["gather"] == grass.GATHER_PREPASS:
+                    alg += 4.0 * wl.T * l.r * k
+                    touched += 2.0 * wl.T * (l.m * dy_touched_share(l.m, l.r) + l.r) * k
             sec = per_kernel["gather"]["ms"] * 1e-3
             hbm["gather"] = {"gbs": alg / sec / 1e9, "touched_gbs": touched / sec / 1e9,
                              "algorithmic_bytes": alg, "touched_bytes": touched}
