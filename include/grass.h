@@ -310,6 +310,7 @@ int grass_layer_step(const grass_step_t* step, void* stream);
  * grass_select, the optional state reset, then grass_layer_step on the rows just selected.
  * step->idx[0] and step->rho[0] (both required) are written by the selection; norms [m] is written.
  * reset_state != 0: M and V are taken as zero without being read (step->step should be 1).
+ * Errors of any part, a projection workspace that is too small included, are returned before the first launch.
  * A small gradient (fewer than 120 output tiles) is formed in norm_ws on the way to its norms, where that
  * is cheaper (grass_refresh_keeps_gradient returns 1 and norm_ws must hold
  * grass_refresh_workspace_bytes): G_C is then its selected rows times rho, and the projection, which would
