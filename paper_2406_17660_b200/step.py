@@ -104,10 +104,9 @@ class GrassLayer:
             dY, X = X, dY        # select columns of X, contract with dY: G_C^T = P^T (X^T dY)
         refresh = self.t % self.K == 0
         if self.fused_update and not (refresh and self._own_refresh()):
+            step = 1 if refresh and self.reset_state else self.adam_step + 1
             if refresh:
-                if self.reset_state:
-                    self.adam_step = 0
-                self._refresh_step(dY, X, self, self.adam_step + 1)
+                self._refresh_step(dY, X, self, step)
             else:
                 call = self._call
                 if call is None:
@@ -115,9 +114,8 @@ class GrassLayer:
                 call.state(0, self.idx, self.rho, self.Gc, self.M, self.V, self.U if self.keep_U else None,
                            self.W, self.side == "cols")
                 call.inputs(0, dY, X)
-                call.launch(1, self.ws.project_ws, self.lr, self.beta1, self.beta2, self.eps,
-                            self.adam_step + 1, self.alpha)
-            self.adam_step += 1
+                call.launch(1, self.ws.project_ws, self.lr, self.beta1, self.beta2, self.eps, step, self.alpha)
+            self.adam_step = step              # (a call that was refused has changed nothing)
             self.t += 1
             return
         if refresh:
@@ -178,12 +176,10 @@ class GrassLayerGroup:
             # the dense gradient that the norms need may already hold the selected rows
             kept = all(l.fused_update and not l._own_refresh() for l in ls) and B.grass_refresh_keeps_gradient(
                 dYs[0].shape[0], first.m, first.n, first.r, B.BF16)
-            for l, dY, X in zip(ls, dYs, Xs):
-                if not kept:
+            if not kept:
+                for l, dY, X in zip(ls, dYs, Xs):
                     l.refresh(dY, X)
-                elif l.reset_state:
-                    l.adam_step = 0
-        step = first.adam_step + 1
+        step = 1 if kept and first.reset_state else first.adam_step + 1
         if kept:
             for l, dY, X in zip(ls, dYs, Xs):
                 l._refresh_step(dY, X, first, step)
@@ -197,5 +193,5 @@ class GrassLayerGroup:
         else:
             self._call.launch(len(ls), self.ws, first.lr, first.beta1, first.beta2, first.eps, step, first.alpha)
         for l in ls:
-            l.adam_step += 1
+            l.adam_step = 1 if kept and l.reset_state else l.adam_step + 1
             l.t += 1

@@ -249,3 +249,25 @@ def test_a_groups_buffers_are_looked_at_again_after_they_were_refused(calls):
     l.W.data = torch.zeros_like(l.W)                 # the same tensor, other memory
     group.step(dYs, Xs)
     assert calls[-1][1]["W"][1] == l.W.data_ptr()
+
+
+@pytest.mark.parametrize("grouped", [False, True])
+def test_a_refused_refresh_leaves_the_counters(calls, monkeypatch, grouped):
+    layers = [layer() for _ in range(2 if grouped else 1)]
+    for l in layers:
+        l.t, l.adam_step = 4, 9
+    stepper = grass.step.GrassLayerGroup(layers, T, device="cpu") if grouped else layers[0]
+    args = (bf16(2, T, M), bf16(2, T, N)) if grouped else (bf16(1, T, M)[0], bf16(1, T, N)[0])
+    library, entry = type(B.load_library()), "grass_refresh_step"
+    good = library.__dict__[entry]
+    monkeypatch.setattr(library, entry, staticmethod(lambda step, refresh, stream: 5))
+    with pytest.raises(grass.GrassError):
+        for l in layers:
+            l._call = None
+        stepper.step(*args)
+    assert [(l.t, l.adam_step) for l in layers] == [(4, 9)] * len(layers)
+    monkeypatch.setattr(library, entry, good)
+    for l in layers:
+        l._call = None
+    stepper.step(*args)
+    assert [(l.t, l.adam_step) for l in layers] == [(5, 1)] * len(layers) and calls[-1][1]["step"] == 1
