@@ -463,14 +463,8 @@ def grass_refresh_keeps_gradient(T: int, m: int, n: int, r: int, dt: int) -> boo
 
 
 _data_ptr = torch.Tensor.data_ptr
+_F32, _I32 = torch.float32, torch.int32
 _CODES = {torch.float32: F32, torch.bfloat16: BF16}
-
-
-def _pitch(shape, stride):
-    """_ld from a tensor's shape and stride."""
-    if len(shape) != 2 or stride[1] != 1:
-        raise ValueError("expected a 2-D tensor with unit inner stride")
-    return stride[0] if shape[0] > 1 else max(stride[0], shape[1])
 
 
 class LayerStepCall:
@@ -495,31 +489,32 @@ class LayerStepCall:
     def state(self, g, idx, rho, Gc, M, V, U, W, cols=False):
         """Layer g's selection, state and weights; layer 0 sets sizes, pitches and W's dtype.
         cols: idx selects columns of W, whose rows the state runs along."""
-        f32 = torch.float32
-        if not (M.dtype is f32 and V.dtype is f32 and Gc.dtype is f32 and idx.dtype is torch.int32
-                and (rho is None or rho.dtype is f32) and (U is None or U.dtype is f32)):
+        if not (M.dtype is _F32 and V.dtype is _F32 and Gc.dtype is _F32 and idx.dtype is _I32
+                and (rho is None or rho.dtype is _F32) and (U is None or U.dtype is _F32)):
             raise TypeError("Gc, M, V, U and rho must be float32 and idx int32")
         if not (M.is_cuda and V.is_cuda and Gc.is_cuda and W.is_cuda and idx.is_cuda
                 and (rho is None or rho.is_cuda) and (U is None or U.is_cuda)):
             raise TypeError("a layer step takes CUDA tensors")
-        shape, stride, wshape = M.shape, M.stride(), W.shape
+        shape, stride, wshape, wstride = M.shape, M.stride(), W.shape, W.stride()
         r, n = shape
         k = 1 if cols else 0
-        if V.shape != shape or Gc.shape != shape or wshape[1 - k] != n or (U is not None and U.shape != shape):
+        if V.shape != shape or Gc.shape != shape or len(wshape) != 2 or wshape[1 - k] != n or \
+                (U is not None and U.shape != shape):
             raise ValueError("Gc, M, V and U must be r x n and W m x n")
         if idx.numel() < r or not idx.is_contiguous() or \
                 (rho is not None and (rho.numel() < r or not rho.is_contiguous())):
             raise ValueError("idx and rho must hold one value per selected row, next to one another")
-        ldm = _pitch(shape, stride)
+        if stride[1] != 1 or wstride[1] != 1:
+            raise ValueError("expected a 2-D tensor with unit inner stride")
+        ldm = stride[0] if r > 1 else max(stride[0], n)
+        ldw = wstride[0] if wshape[0] > 1 else max(wstride[0], wshape[1])
         if (V.stride() != stride and _ld(V) != ldm) or \
                 (U is not None and U.stride() != stride and _ld(U) != ldm):
             raise ValueError("M, V and U must share one row pitch")
         code = _CODES.get(W.dtype)
         if code is None:
             raise TypeError(f"unsupported dtype {W.dtype}")
-        gstride = Gc.stride()
-        own = (r, n, wshape[k], code, ldm if gstride == stride else _pitch(shape, gstride), ldm,
-               _pitch(wshape, W.stride()), k)
+        own = (r, n, wshape[k], code, ldm if Gc.stride() == stride else _ld(Gc), ldm, ldw, k)
         if g == 0:
             a = self.args
             self._own = own
@@ -551,6 +546,8 @@ class LayerStepCall:
         now = (dY.shape, X.shape, dY.stride(), X.stride(), dY.dtype, X.dtype)
         if g == 0:
             yshape, xshape, ystride, xstride, dt, dt2 = self._now = now
+            if len(yshape) != 2 or len(xshape) != 2:
+                raise ValueError("expected a 2-D tensor with unit inner stride")
             if yshape[0] != xshape[0] or dt is not dt2:
                 raise ValueError("dY and X must share the token dimension and dtype")
             _, n, m = self._own[:3]
@@ -559,8 +556,11 @@ class LayerStepCall:
             code = _CODES.get(dt)
             if code is None:
                 raise TypeError(f"unsupported dtype {dt}")
-            a = self.args
-            a.T, a.dt, a.lddy, a.ldx = xshape[0], code, _pitch(yshape, ystride), _pitch(xshape, xstride)
+            if ystride[1] != 1 or xstride[1] != 1:
+                raise ValueError("expected a 2-D tensor with unit inner stride")
+            a, T = self.args, xshape[0]
+            a.T, a.dt = T, code
+            a.lddy, a.ldx = (ystride[0], xstride[0]) if T > 1 else (max(ystride[0], m), max(xstride[0], n))
         elif now != self._now and not (             # (one token has no pitch)
                 now[0][0] == 1 and now[:2] == self._now[:2] and now[4:] == self._now[4:]
                 and now[2][1] == now[3][1] == 1):
@@ -584,7 +584,7 @@ class LayerStepCall:
                 norms, norm_ws, select_ws) -> None:
         """grass_refresh_step on layer 0."""
         self._scalars(1, ws, (lr, beta1, beta2, eps, alpha), step)
-        if norms.dtype is not torch.float32 or not norms.is_cuda:
+        if norms.dtype is not _F32 or not norms.is_cuda:
             raise TypeError("norms must be a CUDA tensor of torch.float32")
         if norms.numel() < self.args.m:
             raise ValueError("norms must hold one value per row")

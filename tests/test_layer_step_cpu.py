@@ -271,3 +271,34 @@ def test_a_refused_refresh_leaves_the_counters(calls, monkeypatch, grouped):
         l._call = None
     stepper.step(*args)
     assert [(l.t, l.adam_step) for l in layers] == [(5, 1)] * len(layers) and calls[-1][1]["step"] == 1
+
+
+@pytest.mark.parametrize("dY,X", [
+    (gpu(T, M, M, dtype=torch.bfloat16), gpu(T, N, dtype=torch.bfloat16)),
+    (gpu(T, M, dtype=torch.bfloat16), gpu(T, N, N, dtype=torch.bfloat16)),
+    (gpu(M, T, dtype=torch.bfloat16).T, gpu(T, N, dtype=torch.bfloat16)),
+    (gpu(T, 2 * M, dtype=torch.bfloat16)[:, ::2], gpu(T, N, dtype=torch.bfloat16)),
+    (gpu(T, M, dtype=torch.bfloat16), gpu(T, N)), (gpu(T, M, dtype=torch.float16), gpu(T, N, dtype=torch.float16)),
+    (gpu(T, M, dtype=torch.bfloat16), gpu(T + 1, N, dtype=torch.bfloat16)), (gpu(T, M - 1, dtype=torch.bfloat16),) * 2,
+    (torch.zeros(T, M, dtype=torch.bfloat16), gpu(T, N, dtype=torch.bfloat16)),
+], ids=str)
+def test_inputs_of_another_form_are_refused(calls, dY, X):
+    call = B.LayerStepCall()
+    call.state(0, **buffers())
+    with pytest.raises((ValueError, TypeError)):
+        call.inputs(0, dY, X)
+
+
+def test_pitches_reach_the_call(calls):
+    wide = buffers()
+    for name, pad in (("M", 3), ("V", 3), ("U", 3), ("Gc", 5)):
+        wide[name] = gpu(R, N + pad)[:, :N]
+    wide["W"] = gpu(M, N + 8, dtype=torch.bfloat16)[:, :N]
+    call = B.LayerStepCall()
+    call.state(0, **wide)
+    call.inputs(0, gpu(T, M + 16, dtype=torch.bfloat16)[:, :M], gpu(T, N + 24, dtype=torch.bfloat16)[:, :N])
+    a = call.args
+    assert (a.ldstate, a.ldgc, a.ldw, a.lddy, a.ldx) == (N + 3, N + 5, N + 8, M + 16, N + 24)
+    for name in ("M", "W", "Gc"):
+        with pytest.raises(ValueError):
+            B.LayerStepCall().state(0, **dict(buffers(), **{name: gpu(*wide[name].shape[::-1], dtype=wide[name].dtype).T}))
