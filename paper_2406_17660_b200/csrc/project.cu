@@ -912,13 +912,16 @@ int project_bf16(int count, const void* const* dY, int64_t lddy, const void* con
   }
   if (plan.gather == kOptPrepass) {
     ProfileScope prof(GRASS_K_GATHER, s);
-    const int ni = plan.r_pad >= 256 ? 8 : plan.r_pad / 32;   // r_pad is a multiple of 64
+    const int ni = plan.r_pad > 128 ? 8 : plan.r_pad / 32;   // r_pad is a multiple of 64
     dim3 ggrid(static_cast<unsigned>((plan.r_pad + 32 * ni - 1) / (32 * ni)),
                static_cast<unsigned>((T + kGatherTokens - 1) / kGatherTokens),
                static_cast<unsigned>(count));
-    auto kernel = sparse_pick(m, r) ? gather_cols_kernel<true> : gather_cols_kernel<false>;
+    const bool sparse = sparse_pick(m, r);
+    auto kernel = ni == 8   ? sparse ? gather_cols_kernel<8, true> : gather_cols_kernel<8, false>
+                  : ni == 4 ? sparse ? gather_cols_kernel<4, true> : gather_cols_kernel<4, false>
+                            : sparse ? gather_cols_kernel<2, true> : gather_cols_kernel<2, false>;
     GRASS_CUDA_TRY(launch_kernel(kernel, ggrid, kGatherThreads, 0, s, dependent, gg, lddy,
-                                 static_cast<int>(T), static_cast<int>(m), r, plan.r_pad, ni, status));
+                                 static_cast<int>(T), static_cast<int>(m), r, plan.r_pad, status));
     dependent = true;
   }
 

@@ -788,28 +788,30 @@ struct GatherGroup {
   __nv_bfloat16* Ag[kTcMaxGroup];
 };
 
-// A warp owns one token at a time and 32 * ni consecutive j: lane l loads
-// j = jb + 32 i + l for i < ni, so one load instruction covers 32 neighbouring
-// selected columns (ascending idx: as few 32-byte sectors as the selection
-// allows) and one store instruction writes 64 contiguous bytes of Ag.
-template <bool SPARSE>
+// A warp owns TU tokens at a time and 32 NI consecutive j: lane l loads j = jb + 32 i + l for i < NI, so one
+// load instruction covers 32 neighbouring selected columns (ascending idx: as few 32-byte sectors as the
+// selection allows) and one store instruction writes 64 contiguous bytes of Ag.  Bound by HBM where rows are long and by
+// loads in flight where they are short: a lane has 16 of them out at r_pad >= 128, whatever NI is, unconditionally
+// (clamped, the value discarded at the store: under a per-lane condition the warp would wait for each).  One token at a
+// time, 4 loads at r = 128, a step took 65.7 us where it takes 57.3 now (T = 65536, 512 x 1376); 29.2 and 25.6
+// (T = 22790, 359 x 1024).
+template <int NI, bool SPARSE>
 __global__ void __launch_bounds__(kGatherThreads)
-gather_cols_kernel(const GatherGroup grp, long long lddy, int T, int m, int r, int r_pad, int ni,
-                   int* status) {
+gather_cols_kernel(const GatherGroup grp, long long lddy, int T, int m, int r, int r_pad, int* status) {
+  constexpr int TU = 16 / NI < kGatherTokens / (kGatherThreads / 32) ? 16 / NI : kGatherTokens / (kGatherThreads / 32);
   grid_dep_launch();        // the blocks of the GEMM find room only when the last of these run
   grid_dep_wait();
   // blockIdx.z = layer of the group
-  const __nv_bfloat16* dY = grp.dY[blockIdx.z];
   const int32_t* idx = grp.idx[blockIdx.z];
-  __nv_bfloat16* Ag = grp.Ag[blockIdx.z];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int jb = blockIdx.x * (32 * ni);
-  int rows[8];
+  const int jb = blockIdx.x * (32 * NI);
+  const int live = (r - jb + 31) / 32;      // groups of 32 columns that hold any
+  int rows[NI];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
+  for (int i = 0; i < NI; ++i) {
     const int j = jb + 32 * i + lane;
     int row = -1;
-    if (i < ni && j < r) {
+    if (j < r) {
       row = ptx::ld_s32(idx + j);
       if (row < 0 || row >= m) {
         record_status(status, GRASS_ERR_INVALID_ARG, row);
@@ -818,20 +820,32 @@ gather_cols_kernel(const GatherGroup grp, long long lddy, int T, int m, int r, i
     }
     rows[i] = row;
   }
-  const unsigned short* src = reinterpret_cast<const unsigned short*>(dY);
-  unsigned short* dst = reinterpret_cast<unsigned short*>(Ag);
+  const unsigned short* src = reinterpret_cast<const unsigned short*>(grp.dY[blockIdx.z]);
+  unsigned short* dst = reinterpret_cast<unsigned short*>(grp.Ag[blockIdx.z]) + jb + lane;
   const int t_begin = blockIdx.y * kGatherTokens;
   const int t_end = t_begin + kGatherTokens < T ? t_begin + kGatherTokens : T;
-#pragma unroll 2
-  for (int t = t_begin + warp; t < t_end; t += kGatherThreads / 32) {
-    const unsigned short* line = src + static_cast<long long>(t) * lddy;
-    unsigned short v[8];
+#pragma unroll 1
+  for (int t = t_begin + warp; t < t_end; t += TU * (kGatherThreads / 32)) {
+    unsigned short v[TU][NI];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = rows[i] >= 0 ? ptx::ld_nc_na_u16<SPARSE>(line + rows[i]) : 0;
-    unsigned short* out = dst + static_cast<long long>(t) * r_pad + jb + lane;
+    for (int u = 0; u < TU; ++u) {
+      const int tok = t + u * (kGatherThreads / 32);
+      const unsigned short* line = src + static_cast<long long>(tok < t_end ? tok : t_end - 1) * lddy;
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
-      if (i < ni && jb + 32 * i + lane < r_pad) out[32 * i] = v[i];
+      for (int i = 0; i < NI; ++i) {
+        v[u][i] = 0;
+        if (i < live) v[u][i] = ptx::ld_nc_na_u16<SPARSE>(line + max(rows[i], 0));
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < TU; ++u) {
+      const int tok = t + u * (kGatherThreads / 32);
+      if (tok >= t_end) break;
+      unsigned short* out = dst + static_cast<long long>(tok) * r_pad;
+#pragma unroll
+      for (int i = 0; i < NI; ++i)
+        if (jb + 32 * i + lane < r_pad) out[32 * i] = rows[i] >= 0 ? v[u][i] : 0;
+    }
   }
 }
 

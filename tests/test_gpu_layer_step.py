@@ -271,3 +271,25 @@ def test_regular_steps_at_full_size(count, T, m, n, r):
         assert rel(l.Gc[js], want) <= 1e-4
         assert float((l.Gc[js] - want).abs().max() / want.abs().max()) <= 1e-4
     check_update(layers, before, 1)
+
+
+@pytest.mark.parametrize("T", [1, 31, 65, 200])
+@pytest.mark.parametrize("r", [1, 64, 65, 128, 129, 192, 257, 320])
+@pytest.mark.parametrize("m", [330, 3400], ids=["dense", "sparse"])
+def test_the_separate_gather_copies_what_the_cooperative_one_does(T, r, m):
+    """Widths and token counts at which the separate gather has lanes, column groups or tokens to spare: the operand,
+    hence G_C, has the bits of the cooperative gather."""
+    n = 136
+    dY, X, _ = inputs(T, m, n)
+    idx = rows_of(m, r)
+    out = []
+    for gather in (grass.binding.GATHER_PREPASS, grass.binding.GATHER_COOPERATIVE):
+        opts = dict(gather=gather, token_slices=1, cta_pair=1, n_blocks_per_cta=1)
+        ws = torch.empty(grass.grass_project_plan(1, T, m, n, r, opts)["workspace_bytes"], dtype=torch.uint8, device=DEV)
+        ws.fill_(0x7f)
+        Gc = torch.empty((r, n), device=DEV)
+        grass.binding.grass_project_grad_ex([dY], [X], [idx], [None], r, [Gc], ws, opts)
+        out.append(Gc)
+    grass.grass_device_status()
+    want = dY[:, idx.long()].double().T @ X.double()
+    assert torch.equal(*out) and rel(out[0], want) <= 1e-5
