@@ -48,8 +48,8 @@ struct ProfileScope {
 // Programmatic dependent launch.  A library call is a chain of short kernels; the second and later
 // ones are launched with this attribute, so that their blocks are placed and run their prologue
 // while the kernel before drains, and wait in grid_dep_wait() for its results.  The first kernel of
-// a call is an ordinary launch: everything enqueued before the call has completed when it starts,
-// and each later kernel waits before it touches memory, so completion is transitive along the chain.
+// a call is an ordinary launch: everything enqueued before the call has completed when it starts, and each later
+// kernel waits before it writes memory or reads what the call writes, so completion is transitive along the chain.
 // A kernel that something follows lets it in with grid_dep_launch(), late enough that the waiting
 // blocks do not hold an SM that another stream could use.
 // What an earlier kernel of the call writes (G_C, partials, norms, idx, rho, the gathered operand) is

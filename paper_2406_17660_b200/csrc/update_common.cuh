@@ -68,6 +68,7 @@ struct UpdateCall {
   int split_k;
   bool part_by_row, reset;
   bool dependent;           // follows another kernel of the same call (common.cuh)
+  bool early;               // .. which writes only the gradient: all else may be read before it has finished
   float alpha;
   AdamScalars a;
 };
