@@ -467,11 +467,27 @@ _F32, _I32 = torch.float32, torch.int32
 _CODES = {torch.float32: F32, torch.bfloat16: BF16}
 
 
+_SCAN = None
+
+
+def _accepted():
+    """accepted() of the built module (csrc/scan.cpp)."""
+    global _SCAN
+    if _SCAN is None:
+        try:
+            from ._scan import accepted
+        except ImportError as e:
+            raise RuntimeError("the _scan module is missing: build it with `python -m paper_2406_17660_b200.build`") from e
+        _SCAN = accepted
+    return _SCAN
+
+
 class LayerStepCall:
     """A grass_step_t and what fills it: state() for the buffers a layer owns, inputs() for what
-    arrives anew with every call.  Both check and marshal everything each time they are called; a
-    step of a small layer takes the GPU no longer than this takes the host, so every tensor
-    attribute is read once."""
+    arrives anew with every call.  Both look at everything each time they are called; a step of a small layer takes
+    the GPU no longer than that takes the host.  So a native scan goes first: tensors that are alike in all but
+    their addresses to the ones that the checks let through last need only their addresses put in place (state()
+    of a layer 2.7 -> 0.2 us, inputs() 1.2 -> 0.1)."""
 
     def __init__(self):
         self.args = a = LayerStep()
@@ -482,6 +498,14 @@ class LayerStepCall:
         lib = load_library()
         self._launch, self._launch_refresh = lib.grass_layer_step, lib.grass_refresh_step
         self._now = self._held = self._pointers = None
+        self._accepted = _accepted()
+        self._at = ctypes.addressof(a) + LayerStep.dY.offset     # of the pointers: nine fields of MAX_GROUP each
+        self._forget()
+
+    def _forget(self):
+        """What the checks let through last, as the scan describes it: per layer with and without cols, and inputs."""
+        self._alike = ([None] * MAX_GROUP, [None] * MAX_GROUP)
+        self._alike_inputs = None
 
     def __reduce__(self):
         return (LayerStepCall, ())       # a copied layer marshals its own buffers anew
@@ -489,6 +513,10 @@ class LayerStepCall:
     def state(self, g, idx, rho, Gc, M, V, U, W, cols=False):
         """Layer g's selection, state and weights; layer 0 sets sizes, pitches and W's dtype.
         cols: idx selects columns of W, whose rows the state runs along."""
+        k = 1 if cols else 0
+        seen = self._accepted(self._at + 8 * (2 * MAX_GROUP + g), self._alike[k][g], idx, rho, Gc, M, V, U, W)
+        if seen is True:
+            return
         if not (M.dtype is _F32 and V.dtype is _F32 and Gc.dtype is _F32 and idx.dtype is _I32
                 and (rho is None or rho.dtype is _F32) and (U is None or U.dtype is _F32)):
             raise TypeError("Gc, M, V, U and rho must be float32 and idx int32")
@@ -497,7 +525,6 @@ class LayerStepCall:
             raise TypeError("a layer step takes CUDA tensors")
         shape, stride, wshape, wstride = M.shape, M.stride(), W.shape, W.stride()
         r, n = shape
-        k = 1 if cols else 0
         if V.shape != shape or Gc.shape != shape or len(wshape) != 2 or wshape[1 - k] != n or \
                 (U is not None and U.shape != shape):
             raise ValueError("Gc, M, V and U must be r x n and W m x n")
@@ -526,6 +553,9 @@ class LayerStepCall:
         sr[g] = None if rho is None else rho.data_ptr()
         sg[g], sm[g], sv[g], sw[g] = Gc.data_ptr(), M.data_ptr(), V.data_ptr(), W.data_ptr()
         su[g] = None if U is None else U.data_ptr()
+        if g == 0:
+            self._forget()                 # the other layers and the inputs are compared with layer 0
+        self._alike[k][g] = seen
 
     def layers_are(self, owns):
         """Whether the tensors that state() was given (all layers', as in the last layers_were()) lie where they
@@ -541,6 +571,9 @@ class LayerStepCall:
 
     def inputs(self, g, dY, X):
         """Layer g's dY (T x m) and X (T x n); after state(0, ..)."""
+        seen = self._accepted(self._at + 8 * g, self._alike_inputs, dY, X)
+        if seen is True:
+            return
         if not (dY.is_cuda and X.is_cuda):
             raise TypeError("a layer step takes CUDA tensors")
         now = (dY.shape, X.shape, dY.stride(), X.stride(), dY.dtype, X.dtype)
@@ -561,6 +594,7 @@ class LayerStepCall:
             a, T = self.args, xshape[0]
             a.T, a.dt = T, code
             a.lddy, a.ldx = (ystride[0], xstride[0]) if T > 1 else (max(ystride[0], m), max(xstride[0], n))
+            self._alike_inputs = seen
         elif now != self._now and not (             # (one token has no pitch)
                 now[0][0] == 1 and now[:2] == self._now[:2] and now[4:] == self._now[4:]
                 and now[2][1] == now[3][1] == 1):

@@ -2,8 +2,9 @@
 
     python -m paper_2406_17660_b200.build
 
-Produces paper_2406_17660_b200/libgrass_b200.so next to this file.  nvcc
-cross-compiles without a GPU, so this runs on any box with the CUDA toolkit.
+Produces libgrass_b200.so (the CUDA library, nvcc) and _scan.so (the binding's scan of torch tensors,
+g++ against torch's headers) next to this file.  nvcc cross-compiles without a GPU, so this runs on any
+box with the CUDA toolkit.
 """
 from __future__ import annotations
 
@@ -11,11 +12,13 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libgrass_b200.so")
+SCAN = os.path.join(HERE, "_scan.so")
 SOURCES = ["common.cu", "row_norms.cu", "select.cu", "project.cu", "adam.cu", "scatter.cu",
            "adam_scatter.cu", "selftest.cu"]
 
@@ -28,12 +31,23 @@ def _nvcc() -> str:
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not (os.path.exists(LIB) and os.path.exists(SCAN)):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(SCAN))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)]
     deps += [os.path.join(ROOT, "include", f) for f in os.listdir(os.path.join(ROOT, "include"))]
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def _scan_command() -> list:
+    import torch
+    from torch.utils.cpp_extension import include_paths
+    cmd = [shutil.which("g++") or "g++", "-O2", "-std=c++17", "-shared", "-fPIC",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+    for path in include_paths():
+        cmd += ["-isystem", path]
+    return cmd + ["-I", sysconfig.get_paths()["include"], "-o", SCAN, os.path.join(CSRC, "scan.cpp"), "-L",
+                  os.path.join(os.path.dirname(torch.__file__), "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10"]
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -50,6 +64,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
         raise RuntimeError("nvcc failed building libgrass_b200.so")
     if verbose:
         sys.stderr.write(res.stderr)
+    res = subprocess.run(_scan_command(), capture_output=True, text=True)
+    if res.returncode != 0:
+        sys.stderr.write(res.stdout + res.stderr)
+        raise RuntimeError("g++ failed building _scan.so")
     return LIB
 
 

@@ -1,0 +1,81 @@
+// _scan: what a layer-step's tensors are, read in one call.
+//
+// A step of a small layer takes the GPU about as long as it takes the host to look through its nine tensors from
+// Python (4 us: dtype, device, shape, strides and address are an attribute access each).  accepted() reads all of that
+// for a call's tensors, compares it with what the full checks last let through, and only if nothing differs writes the
+// addresses to where the call expects them (0.2 us).  Nothing is remembered by a tensor's identity or address.
+#define PY_SSIZE_T_CLEAN
+#include <Python.h>
+#include <torch/csrc/autograd/python_variable.h>
+
+#include <cstdint>
+#include <cstring>
+
+namespace {
+
+struct Seen {
+  int64_t kind;                      // 0: None
+  int64_t dtype, device, dim, numel, contiguous, sizes[2], strides[2];
+};
+constexpr int kMost = 8;
+
+// False: not a plain tensor that has storage (the caller's own checks decide).
+bool look(PyObject* o, Seen& s, void*& at) {
+  std::memset(&s, 0, sizeof(s));
+  at = nullptr;
+  if (o == Py_None) return true;
+  if (!THPVariable_CheckExact(o)) return false;
+  const at::Tensor& t = THPVariable_Unpack(o);
+  if (!t.has_storage() || t.layout() != at::kStrided || t.dim() > 2) return false;
+  s.kind = 1;
+  s.dtype = static_cast<int64_t>(t.scalar_type());
+  s.device = static_cast<int64_t>(t.device().type()) * 256 + t.device().index();
+  s.dim = t.dim();
+  s.numel = t.numel();
+  s.contiguous = t.is_contiguous();
+  for (int64_t d = 0; d < s.dim; ++d) {
+    s.sizes[d] = t.size(d);
+    s.strides[d] = t.stride(d);
+  }
+  at = t.data_ptr();
+  return true;
+}
+
+// accepted(address, before, tensor or None, ...): True, and tensor i's address is at address + 64 i, if the tensors are
+// alike in all but their addresses to those that `before` describes; else their description, or None where there is none.
+PyObject* accepted(PyObject*, PyObject* const* args, Py_ssize_t n) {
+  if (n < 3 || n - 2 > kMost) {
+    PyErr_SetString(PyExc_TypeError, "accepted(address, before, tensor, ...) takes one to eight tensors");
+    return nullptr;
+  }
+  const unsigned long long address = PyLong_AsUnsignedLongLong(args[0]);
+  if (PyErr_Occurred()) return nullptr;
+  Seen seen[kMost];
+  void* at[kMost];
+  const Py_ssize_t count = n - 2;
+  try {
+    for (Py_ssize_t i = 0; i < count; ++i)
+      if (!look(args[i + 2], seen[i], at[i])) Py_RETURN_NONE;
+  } catch (...) {                    // (a tensor that will not say where it is)
+    Py_RETURN_NONE;
+  }
+  const Py_ssize_t bytes = count * static_cast<Py_ssize_t>(sizeof(Seen));
+  const char* now = reinterpret_cast<const char*>(seen);
+  PyObject* before = args[1];
+  if (PyBytes_Check(before) && PyBytes_GET_SIZE(before) == bytes &&
+      std::memcmp(PyBytes_AS_STRING(before), now, bytes) == 0) {
+    for (Py_ssize_t i = 0; i < count; ++i) *reinterpret_cast<void**>(address + 64 * i) = at[i];
+    Py_RETURN_TRUE;
+  }
+  return PyBytes_FromStringAndSize(now, bytes);
+}
+
+PyMethodDef methods[] = {
+    {"accepted", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(accepted)), METH_FASTCALL,
+     "whether tensors are alike to those let through before; writes their addresses if so"},
+    {nullptr, nullptr, 0, nullptr}};
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_scan", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__scan() { return PyModule_Create(&module); }

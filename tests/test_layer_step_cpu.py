@@ -302,3 +302,46 @@ def test_pitches_reach_the_call(calls):
     for name in ("M", "W", "Gc"):
         with pytest.raises(ValueError):
             B.LayerStepCall().state(0, **dict(buffers(), **{name: gpu(*wide[name].shape[::-1], dtype=wide[name].dtype).T}))
+
+
+def test_the_scan_takes_only_tensors_alike_to_those_let_through():
+    """accepted(): addresses are written only where shape, strides, dtype, device and which are None all agree; what is no
+    plain tensor is left to the checks."""
+    accepted = B._accepted()
+    at = (ctypes.c_uint64 * (8 * 3))()
+    where = ctypes.addressof(at)
+    x, y = torch.zeros(4, 6), torch.zeros(8, dtype=torch.int32)
+    seen = accepted(where, None, x, None, y)
+    assert isinstance(seen, bytes) and not any(at)
+    other = torch.ones(4, 6), None, torch.ones(8, dtype=torch.int32)
+    assert accepted(where, seen, *other) is True
+    assert (at[0], at[8], at[16]) == (other[0].data_ptr(), 0, other[2].data_ptr())
+    was = list(at)
+    for bad in ((x.T.contiguous().T, None, y), (torch.zeros(4, 7)[:, :6], None, y), (x.double(), None, y),
+                (x, y, None), (x, x, y), (x, None, y[:7]), (x, None, torch.zeros(16, dtype=torch.int32)[::2]),
+                (x.to("meta"), None, y)):
+        assert accepted(where, seen, *bad) is not True and list(at) == was
+    for odd in (gpu(4, 6), 3, torch.zeros(2, 2, 2), torch.zeros(4, 6).to_sparse()):
+        assert accepted(where, seen, odd, None, y) is None and list(at) == was
+
+
+def test_a_scanned_call_is_checked_again_when_layer_0_changes(calls, monkeypatch):
+    """Other layers and the inputs go with layer 0's sizes: what was let through with one layer 0 is not with another."""
+    plain = {k: torch.zeros(v.shape, dtype=v.dtype) for k, v in buffers().items()}
+    monkeypatch.setattr(torch.Tensor, "is_cuda", True)
+    call = B.LayerStepCall()
+    for g in range(2):
+        call.state(g, **plain)
+        call.inputs(g, torch.zeros(T, M, dtype=torch.bfloat16), torch.zeros(T, N, dtype=torch.bfloat16))
+    again = {k: v.clone() for k, v in plain.items()}
+    call.state(1, **again)
+    assert call.args.M[1] == again["M"].data_ptr() and call.args.W[0] == plain["W"].data_ptr()
+    call.state(0, **{k: torch.zeros(v.shape, dtype=v.dtype) for k, v in buffers(r=R - 1).items()})
+    assert call.args.r == R - 1
+    with pytest.raises(ValueError):
+        call.state(1, **again)
+    call.state(0, **{k: torch.zeros(v.shape, dtype=v.dtype) for k, v in buffers(n=N + 8).items()})
+    with pytest.raises(ValueError):
+        call.inputs(0, torch.zeros(T, M, dtype=torch.bfloat16), torch.zeros(T, N, dtype=torch.bfloat16))
+    with pytest.raises(ValueError):
+        call.state(0, **plain, cols=True)
