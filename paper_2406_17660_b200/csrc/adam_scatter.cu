@@ -473,7 +473,7 @@ int launch_cols(const UpdateCall& u, cudaStream_t s) {
   dim3 grid(static_cast<unsigned>(blocks), 1, static_cast<unsigned>(u.count));
   ProfileScope prof(GRASS_K_ADAM_SCATTER, s);
   GRASS_CUDA_TRY(launch_kernel(u.split_k > 0 ? adam_apply_cols_kernel<T, true> : adam_apply_cols_kernel<T, false>,
-                               grid, kThreads, 0, s, u.dependent, u.grp, u.ldgc, u.ldstate, u.m, u.n, u.ldw,
+                               grid, kThreads, 0, s, u.grp, u.ldgc, u.ldstate, u.m, u.n, u.ldw,
                                u.r, u.ld_part, u.split_stride, u.split_k, u.part_by_row, u.reset, u.early, u.alpha,
                                u.a, status));
   return GRASS_OK;
@@ -485,7 +485,7 @@ int launch_narrow(const UpdateCall& u, int* status, cudaStream_t s) {
             static_cast<unsigned>(u.count));
   {
     ProfileScope prof(GRASS_K_ADAM_SCATTER, s);
-    GRASS_CUDA_TRY(launch_kernel(adam_apply_narrow_kernel<T, SPLIT>, grid, kThreads, 0, s, u.dependent,
+    GRASS_CUDA_TRY(launch_kernel(adam_apply_narrow_kernel<T, SPLIT>, grid, kThreads, 0, s,
         u.grp, u.ldgc, u.ldstate, u.m, u.n, u.ldw, u.r, u.ld_part, u.split_stride, u.split_k, u.part_by_row,
         u.reset, u.early, u.alpha, u.a, status));
   }
@@ -509,7 +509,7 @@ int launch_wide(const UpdateCall& u, int* status, cudaStream_t s) {
     ProfileScope prof(GRASS_K_ADAM_SCATTER, s);
     GRASS_CUDA_TRY(launch_kernel(
         vec ? adam_apply_wide_kernel<T, E, true, SPLIT> : adam_apply_wide_kernel<T, E, false, SPLIT>, grid,
-        threads, 0, s, u.dependent, u.grp, u.ldgc, u.ldstate, u.m, u.n, u.ldw, u.r, u.ld_part,
+        threads, 0, s, u.grp, u.ldgc, u.ldstate, u.m, u.n, u.ldw, u.r, u.ld_part,
         u.split_stride, u.split_k, u.part_by_row, u.reset, u.early, u.alpha, u.a, status));
   }
   return GRASS_OK;

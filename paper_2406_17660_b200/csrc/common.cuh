@@ -19,8 +19,8 @@ __device__ __forceinline__ void record_status(int* status, int code, int detail)
 // Device address of the current device's status word (host function, common.cu).
 int* status_word(cudaError_t* err);
 
-// grass_select; dependent: see launch_kernel below (select.cu).
-int select_rows(bool dependent, const float* norms, int64_t m, int32_t r, int method, uint64_t seed,
+// grass_select (select.cu).
+int select_rows(const float* norms, int64_t m, int32_t r, int method, uint64_t seed,
                 uint32_t layer_id, uint32_t epoch, int32_t* idx, float* rho, void* ws, size_t ws_bytes,
                 cudaStream_t s);
 
@@ -45,18 +45,19 @@ struct ProfileScope {
 
 #define GRASS_LAUNCH_CHECK() GRASS_CUDA_TRY(cudaGetLastError())
 
-// Programmatic dependent launch.  A library call is a chain of short kernels; the second and later
-// ones are launched with this attribute, so that their blocks are placed and run their prologue
-// while the kernel before drains, and wait in grid_dep_wait() for its results.  The first kernel of
-// a call is an ordinary launch: everything enqueued before the call has completed when it starts, and each later
-// kernel waits before it writes memory or reads what the call writes, so completion is transitive along the chain.
-// A kernel that something follows lets it in with grid_dep_launch(), late enough that the waiting
+// Programmatic dependent launch.  A library call is a chain of short kernels.  They are launched with this
+// attribute, the first one too, so that their blocks are placed and run their prologue while the kernel before drains, and
+// wait in grid_dep_wait() for its results.  Each waits before it writes memory or reads what an earlier kernel of the
+// call or of the stream writes, so completion is transitive along the chain and along the stream.  (The one exception is
+// UpdateCall::early: by the time those blocks run, the kernel before them has waited itself.)  The kernel that another
+// call's first kernel follows lets it in only by ending.  Eagerly launched steps gained 1 to 2.7 us from the
+// attribute on their first kernel (T = 4096, 1024 x 1024, r = 128: 16.4 -> 13.7).
+// A kernel that something follows in its call lets it in with grid_dep_launch(), late enough that the waiting
 // blocks do not hold an SM that another stream could use.
-// What an earlier kernel of the call writes (G_C, partials, norms, idx, rho, the gathered operand) is
-// still being written when a dependent kernel becomes resident, so it is not constant for that kernel's
-// lifetime: such a kernel reads it with ordinary loads (also ptx::ld_s32, ld_f32), through pointers
-// without __restrict__ and without __ldg, which the compiler could move above grid_dep_wait().  Read-only
-// loads (ld_nc_*) are for inputs of the call.
+// What an earlier kernel writes (inputs made by the program's last kernel, G_C, partials, norms, idx, rho, the gathered
+// operand) is still being written when a dependent kernel becomes resident, so it is not constant for that kernel's
+// lifetime: such a kernel reads it with ordinary loads (also ptx::ld_s32, ld_f32, ld_na_u16), through pointers
+// without __restrict__ and without __ldg, which the compiler could move above grid_dep_wait().
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -67,10 +68,10 @@ inline cudaLaunchAttribute dependent_launch_attr() {
   a.val.programmaticStreamSerializationAllowed = 1;
   return a;
 }
-// dependent: the previous operation on the stream is a kernel of the same library call.
+// For kernels that call grid_dep_wait().
 template <typename... P, typename... A>
 cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                          bool dependent, A&&... args) {
+                          A&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -78,7 +79,7 @@ cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t sm
   cfg.stream = s;
   cudaLaunchAttribute attr = dependent_launch_attr();
   cfg.attrs = &attr;
-  cfg.numAttrs = dependent ? 1 : 0;
+  cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 

@@ -597,7 +597,7 @@ bool make_map(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, in
 
 template <int MB, int NSLAB, bool PAIR, int GATHER>
 int launch_tc_one(dim3 tile_grid, size_t smem, cudaStream_t s, const TcMaps& maps, TcParams p,
-                  int kernel_id, bool dependent) {
+                  int kernel_id) {
   constexpr bool FUSED = GATHER != kGatherNone;   // the variants with eight extra warps
   static bool attr_set[64] = {false};
   static int max_workers[64] = {0};
@@ -640,10 +640,8 @@ int launch_tc_one(dim3 tile_grid, size_t smem, cudaStream_t s, const TcMaps& map
   const int workers = n_tiles < max_workers[dev] && GATHER != kGatherCoop && p.s_long == p.split_k
                           ? static_cast<int>(n_tiles) : max_workers[dev];
   cfg.gridDim = dim3(static_cast<unsigned>(PAIR ? 2 * workers : workers));
-  if (dependent) {
-    attr[1] = dependent_launch_attr();
-    cfg.numAttrs = 2;
-  }
+  attr[1] = dependent_launch_attr();
+  cfg.numAttrs = 2;
   {
     ProfileScope prof(kernel_id, s);
     GRASS_CUDA_TRY(cudaLaunchKernelEx(&cfg, project_tc_kernel<MB, NSLAB, PAIR, GATHER>, maps, p));
@@ -654,10 +652,10 @@ int launch_tc_one(dim3 tile_grid, size_t smem, cudaStream_t s, const TcMaps& map
 // (MB, NSLAB) with MB * 64 * NSLAB <= 512 TMEM columns; pairs need an even NSLAB.
 // gather: kGatherNone / kGatherCta (tiles of at most 128 rows) / kGatherCoop.
 int launch_tc(int MB, int nslab, bool pair, int gather, dim3 grid, size_t smem, cudaStream_t s,
-              const TcMaps& maps, const TcParams& p, int kernel_id, bool dependent) {
+              const TcMaps& maps, const TcParams& p, int kernel_id) {
 #define GRASS_TC_CASE(mb, ns, pr, ga)                                                          \
   if (MB == mb && nslab == ns && pair == pr && gather == ga)                                   \
-    return launch_tc_one<mb, ns, pr, ga>(grid, smem, s, maps, p, kernel_id, dependent)
+    return launch_tc_one<mb, ns, pr, ga>(grid, smem, s, maps, p, kernel_id)
 #define GRASS_TC_BOTH(mb, ns, pr)                                                              \
   GRASS_TC_CASE(mb, ns, pr, kGatherNone);                                                      \
   GRASS_TC_CASE(mb, ns, pr, kGatherCoop)
@@ -753,7 +751,7 @@ int launch_simt(const Fp32Plan& fp, const float* dY, int64_t lddy, const float* 
   const bool xvec = aligned_to(X, 16) && ldx % 4 == 0;
   const bool ovec = aligned_to(out, 16) && ld_out % 4 == 0;
   ProfileScope prof(GRASS_K_PROJECT_FP32, s);
-  GRASS_CUDA_TRY(launch_kernel(project_simt_kernel<TM>, grid, kSimtThreads, simt_smem_bytes(TM), s, false,
+  GRASS_CUDA_TRY(launch_kernel(project_simt_kernel<TM>, grid, kSimtThreads, simt_smem_bytes(TM), s,
                                dY, lddy, X, ldx, T, m, n, idx, rho, r, out, ld_out, fp.tokens_per_split,
                                static_cast<int64_t>(r) * fp.ld_part, avec, xvec, ovec, status));
   return GRASS_OK;
@@ -842,7 +840,7 @@ cudaError_t launch_row_norms(const float* part, long long ld, long long stride, 
   while (threads < 256 && m * threads / 256 < 2 * kSmCount) threads *= 2;
   const int rows = 256 / threads;
   auto kernel = threads < 256 ? splitk_rownorms_kernel<true> : splitk_rownorms_kernel<false>;
-  return launch_kernel(kernel, static_cast<unsigned>((m + rows - 1) / rows), 256, 0, s, true, part, ld, stride,
+  return launch_kernel(kernel, static_cast<unsigned>((m + rows - 1) / rows), 256, 0, s, part, ld, stride,
                        split_k, static_cast<int>(m), static_cast<int>(n), threads, norms);
 }
 
@@ -854,7 +852,7 @@ int project_bf16(int count, const void* const* dY, int64_t lddy, const void* con
                  int64_t T, int64_t m, int64_t n, const int32_t* const* idx,
                  const float* const* rho, int r, float* const* Gc, int64_t ldgc, float* norms,
                  void* ws, size_t ws_bytes, const PlanOpts& opts, cudaStream_t s,
-                 UpdateCall* upd = nullptr, GradParts* keep = nullptr, bool dependent = false) {
+                 UpdateCall* upd = nullptr, GradParts* keep = nullptr) {
   if (count < 1 || count > kTcMaxGroup || (norms != nullptr && count != 1))
     return GRASS_ERR_INVALID_ARG;
   const bool gather = idx != nullptr && idx[0] != nullptr;
@@ -920,9 +918,8 @@ int project_bf16(int count, const void* const* dY, int64_t lddy, const void* con
     auto kernel = ni == 8   ? sparse ? gather_cols_kernel<8, true> : gather_cols_kernel<8, false>
                   : ni == 4 ? sparse ? gather_cols_kernel<4, true> : gather_cols_kernel<4, false>
                             : sparse ? gather_cols_kernel<2, true> : gather_cols_kernel<2, false>;
-    GRASS_CUDA_TRY(launch_kernel(kernel, ggrid, kGatherThreads, 0, s, dependent, gg, lddy,
+    GRASS_CUDA_TRY(launch_kernel(kernel, ggrid, kGatherThreads, 0, s, gg, lddy,
                                  static_cast<int>(T), static_cast<int>(m), r, plan.r_pad, status));
-    dependent = true;
   }
 
   TcParams p;
@@ -962,9 +959,8 @@ int project_bf16(int count, const void* const* dY, int64_t lddy, const void* con
     // queue head and per-chunk counters start at zero for every launch
     p.coop_ctrl = static_cast<int*>(ws);
     const int ints = static_cast<int>(plan.ctrl_bytes / sizeof(int));
-    GRASS_CUDA_TRY(launch_kernel(zero_ctrl_kernel, (ints + 1023) / 1024, 1024, 0, s, dependent,
+    GRASS_CUDA_TRY(launch_kernel(zero_ctrl_kernel, (ints + 1023) / 1024, 1024, 0, s,
                                  p.coop_ctrl, ints));
-    dependent = true;
   }
   p.ld_norm = static_cast<long long>(round_up(static_cast<size_t>(m), 32));
   for (int g = 0; g < kTcMaxGroup; ++g) {
@@ -986,14 +982,13 @@ int project_bf16(int count, const void* const* dY, int64_t lddy, const void* con
   const int kernel_gather = plan.gather == kOptCta ? kGatherCta
                             : plan.gather == kOptCoop ? kGatherCoop : kGatherNone;
   const int rc = launch_tc(plan.MB, plan.r_cta / 64, plan.pair, kernel_gather, grid, plan.smem_bytes,
-                           s, maps, p, gather ? GRASS_K_PROJECT_TC : GRASS_K_PROJECT_TC_DENSE,
-                           dependent);
+                           s, maps, p, gather ? GRASS_K_PROJECT_TC : GRASS_K_PROJECT_TC_DENSE);
   if (rc != GRASS_OK) return rc;
   if (norms != nullptr) {
     ProfileScope prof(GRASS_K_ROW_NORMS, s);
     if (fused_norms)
       GRASS_CUDA_TRY(launch_kernel(norms_finalize_kernel, static_cast<unsigned>((m + 255) / 256), 256, 0, s,
-                                   true, p.norm_part, p.ld_norm, static_cast<int>((n + 31) / 32),
+                                   p.norm_part, p.ld_norm, static_cast<int>((n + 31) / 32),
                                    static_cast<int>(m), norms));
     else
       GRASS_CUDA_TRY(launch_row_norms(part[0], plan.ld_part, p.split_stride, plan.split_k, m, n, norms, s));
@@ -1005,7 +1000,6 @@ int project_bf16(int count, const void* const* dY, int64_t lddy, const void* con
     upd->split_k = plan.split_k > 1 ? plan.split_k : 0;
     upd->ld_part = plan.ld_part;
     upd->split_stride = p.split_stride;
-    upd->dependent = true;
     return launch_update(*upd, s);
   }
   if (plan.split_k > 1) {
@@ -1024,7 +1018,7 @@ int project_bf16(int count, const void* const* dY, int64_t lddy, const void* con
     ProfileScope prof(GRASS_K_SPLITK_REDUCE, s);
     GRASS_CUDA_TRY(launch_kernel(splitk_reduce_kernel,
                                  dim3(static_cast<unsigned>(blocks), static_cast<unsigned>(count)), 256, 0, s,
-                                 true, rg, plan.ld_part, p.split_stride, plan.split_k, r,
+                                 rg, plan.ld_part, p.split_stride, plan.split_k, r,
                                  static_cast<int>(n), ldgc, vec));
   }
   return GRASS_OK;
@@ -1109,7 +1103,6 @@ int project_fp32(const void* dY, int64_t lddy, const void* X, int64_t ldx, int64
     upd->split_k = fp.split > 1 ? fp.split : 0;
     upd->ld_part = fp.ld_part;
     upd->split_stride = static_cast<long long>(r) * fp.ld_part;
-    upd->dependent = true;
     return launch_update(*upd, s);
   }
   if (fp.split > 1) {
@@ -1120,7 +1113,7 @@ int project_fp32(const void* dY, int64_t lddy, const void* X, int64_t ldx, int64
     ProfileScope prof(GRASS_K_SPLITK_REDUCE, s);
     ReduceGroup rg;
     for (int g = 0; g < kTcMaxGroup; ++g) { rg.part[g] = out; rg.rho[g] = rho; rg.Gc[g] = Gc; }
-    GRASS_CUDA_TRY(launch_kernel(splitk_reduce_kernel, static_cast<unsigned>(blocks), 256, 0, s, true, rg,
+    GRASS_CUDA_TRY(launch_kernel(splitk_reduce_kernel, static_cast<unsigned>(blocks), 256, 0, s, rg,
                                  fp.ld_part, static_cast<long long>(r) * fp.ld_part, fp.split, r,
                                  static_cast<int>(n), ldgc, vec));
   }
@@ -1232,8 +1225,7 @@ int project_and_update(const grass_step_t* a, UpdateCall& u, cudaStream_t s, boo
                         a->r, a->Gc[0], a->ldgc, a->ws, a->ws_bytes, s, &u, nullptr, nullptr,
                         refresh ? a->r : 0);
   return project_bf16(a->count, a->dY, a->lddy, a->X, a->ldx, a->T, a->m, a->n, a->idx, a->rho, a->r,
-                      a->Gc, a->ldgc, nullptr, a->ws, a->ws_bytes, refresh ? PlanOpts() : wide_opts(), s, &u,
-                      nullptr, refresh);
+                      a->Gc, a->ldgc, nullptr, a->ws, a->ws_bytes, refresh ? PlanOpts() : wide_opts(), s, &u);
 }
 
 // What the projection of a refresh iteration will refuse, if it has one: asked before the selection
@@ -1323,13 +1315,12 @@ extern "C" int grass_refresh_step(const grass_step_t* a, const grass_refresh_t* 
   rc2 = grad_row_norms(a->dY[0], a->lddy, a->X[0], a->ldx, a->dt, a->T, a->m, a->n, f->norms,
                            f->norm_ws, f->norm_ws_bytes, s, &kept);
   if (rc2 != GRASS_OK) return rc2;
-  rc2 = select_rows(true, f->norms, a->m, a->r, f->method, f->seed, f->layer_id, f->epoch,
+  rc2 = select_rows(f->norms, a->m, a->r, f->method, f->seed, f->layer_id, f->epoch,
                      const_cast<int32_t*>(a->idx[0]), const_cast<float*>(a->rho[0]), f->select_ws,
                      f->select_ws_bytes, s);
   if (rc2 != GRASS_OK) return rc2;
   u.reset = f->reset_state != 0;
   if (kept.split_k == 0) return project_and_update(a, u, s, true);
-  u.dependent = true;
   u.grp.part[0] = kept.part;
   u.ld_part = kept.ld;
   u.split_stride = kept.stride;

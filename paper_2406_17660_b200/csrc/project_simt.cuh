@@ -45,9 +45,9 @@ __device__ __forceinline__ void fma_pair(float2& d, float2 a, float2 b) {
 // avec / xvec: the dense dY / X may be copied 16 bytes at a time; ovec: so may the output.
 template <int TM>
 __global__ void __launch_bounds__(kSimtThreads, TM == 8 ? 2 : 4)
-project_simt_kernel(const float* __restrict__ dY, int64_t lddy, const float* __restrict__ X, int64_t ldx,
-                    int64_t Ttok, int64_t m, int64_t n, const int32_t* __restrict__ idx,
-                    const float* __restrict__ rho, int r, float* __restrict__ Gc, int64_t ldgc,
+project_simt_kernel(const float* dY, int64_t lddy, const float* X, int64_t ldx,
+                    int64_t Ttok, int64_t m, int64_t n, const int32_t* idx,
+                    const float* rho, int r, float* Gc, int64_t ldgc,
                     int64_t tokens_per_split, int64_t split_stride, bool avec, bool xvec, bool ovec,
                     int* status) {
   constexpr int B = simt_tile(TM), BT = kSimtBT, Q = TM / 4;
@@ -57,6 +57,7 @@ project_simt_kernel(const float* __restrict__ dY, int64_t lddy, const float* __r
   const int tid = threadIdx.x;
   const int j0 = blockIdx.y * B;
   const int64_t c0 = static_cast<int64_t>(blockIdx.x) * B;
+  grid_dep_wait();
   // the selected row whose column this thread copies
   int row = -1;
   if (!avec) {

@@ -169,8 +169,8 @@ __device__ __forceinline__ float warp_transpose_sum(float (&x)[32], int lane) {
 // dY[t, rows[i]] for 32 (token, column) pairs per lane in flight, written to the operand matrix.
 // Lane l carries columns col0 + 32 i + l, i < NI; tokens tok0, tok0 + kCoopParts, ...
 template <int NI, bool SPARSE>
-__device__ __forceinline__ void coop_gather_part(const unsigned short* __restrict__ src,
-                                                 long long lddy, unsigned short* __restrict__ dst,
+__device__ __forceinline__ void coop_gather_part(const unsigned short* src,
+                                                 long long lddy, unsigned short* dst,
                                                  int r_pad, int col0, const int (&rows)[8], int tok0,
                                                  int T, int lane, int* publish) {
   constexpr int TU = (32 / NI) < (kCoopChunk / kCoopParts) ? (32 / NI) : (kCoopChunk / kCoopParts);   // tokens per batch of loads
@@ -189,7 +189,7 @@ __device__ __forceinline__ void coop_gather_part(const unsigned short* __restric
       const int tok = tok0 + (k0 + u) * kCoopParts;
       const unsigned short* line = src + static_cast<long long>(tok < T ? tok : T - 1) * lddy;
 #pragma unroll
-      for (int i = 0; i < NI; ++i) v[u][i] = ptx::ld_nc_na_u16<SPARSE>(line + safe[i]);
+      for (int i = 0; i < NI; ++i) v[u][i] = ptx::ld_na_u16<SPARSE>(line + safe[i]);
     }
     if (publish != nullptr) {
       // the previous item's stores (all lanes, program order + warp barrier) become visible
@@ -666,8 +666,8 @@ project_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
             const unsigned short* line = src + static_cast<long long>(tok < p.T ? tok : p.T - 1) * p.lddy;
 #pragma unroll
             for (int a = 0; a < A_SLABS; ++a) {
-              v[k][a][0] = ptx::ld_nc_u16(line + max(rows[a][0], 0));
-              v[k][a][1] = ptx::ld_nc_u16(line + max(rows[a][1], 0));
+              v[k][a][0] = ptx::ld_u16(line + max(rows[a][0], 0));
+              v[k][a][1] = ptx::ld_u16(line + max(rows[a][1], 0));
             }
           }
 #pragma unroll
@@ -834,7 +834,7 @@ gather_cols_kernel(const GatherGroup grp, long long lddy, int T, int m, int r, i
 #pragma unroll
       for (int i = 0; i < NI; ++i) {
         v[u][i] = 0;
-        if (i < live) v[u][i] = ptx::ld_nc_na_u16<SPARSE>(line + max(rows[i], 0));
+        if (i < live) v[u][i] = ptx::ld_na_u16<SPARSE>(line + max(rows[i], 0));
       }
     }
 #pragma unroll

@@ -37,12 +37,12 @@ template <> struct Vec<__nv_bfloat16> {
 
 template <typename T, int TPR, bool VEC>
 __global__ void __launch_bounds__(kThreads)
-row_norms_kernel(const T* __restrict__ G, int64_t m, int64_t n, int64_t ldg,
-                 float* __restrict__ norms) {
+row_norms_kernel(const T* G, int64_t m, int64_t n, int64_t ldg, float* norms) {
   constexpr int ROWS = kThreads / TPR;
   const int lane_in_row = threadIdx.x % TPR;
   const int64_t row = static_cast<int64_t>(blockIdx.x) * ROWS + threadIdx.x / TPR;
   float acc0 = 0.f, acc1 = 0.f, acc2 = 0.f, acc3 = 0.f;
+  grid_dep_wait();
   if (row < m) {
     const T* g = G + row * ldg;
     if (VEC) {
@@ -54,21 +54,21 @@ row_norms_kernel(const T* __restrict__ G, int64_t m, int64_t n, int64_t ldg,
       for (; i + 7 * TPR < nv; i += 8 * TPR) {
         V v[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = __ldg(gv + i + u * TPR);
+        for (int u = 0; u < 8; ++u) v[u] = gv[i + u * TPR];
         acc0 += Vec<T>::sumsq(v[0]) + Vec<T>::sumsq(v[4]);
         acc1 += Vec<T>::sumsq(v[1]) + Vec<T>::sumsq(v[5]);
         acc2 += Vec<T>::sumsq(v[2]) + Vec<T>::sumsq(v[6]);
         acc3 += Vec<T>::sumsq(v[3]) + Vec<T>::sumsq(v[7]);
       }
       for (; i + 3 * TPR < nv; i += 4 * TPR) {
-        V a = __ldg(gv + i), b = __ldg(gv + i + TPR), c = __ldg(gv + i + 2 * TPR),
-          d = __ldg(gv + i + 3 * TPR);
+        V a = gv[i], b = gv[i + TPR], c = gv[i + 2 * TPR],
+          d = gv[i + 3 * TPR];
         acc0 += Vec<T>::sumsq(a);
         acc1 += Vec<T>::sumsq(b);
         acc2 += Vec<T>::sumsq(c);
         acc3 += Vec<T>::sumsq(d);
       }
-      for (; i < nv; i += TPR) acc0 += Vec<T>::sumsq(__ldg(gv + i));
+      for (; i < nv; i += TPR) acc0 += Vec<T>::sumsq(gv[i]);
       for (int64_t c = nv * N + lane_in_row; c < n; c += TPR) {
         float v = to_float(g[c]);
         acc1 += v * v;
@@ -107,12 +107,11 @@ int launch(const void* G, int64_t m, int64_t n, int64_t ldg, float* norms, cudaS
   ProfileScope prof(GRASS_K_ROW_NORMS, s);
 #define GRASS_NORMS_CASE(TPR)                                                                   \
   if (tpr == TPR) {                                                                             \
-    if (vec) row_norms_kernel<T, TPR, true><<<grid, kThreads, 0, s>>>(g, m, n, ldg, norms);     \
-    else     row_norms_kernel<T, TPR, false><<<grid, kThreads, 0, s>>>(g, m, n, ldg, norms);    \
+    GRASS_CUDA_TRY(launch_kernel(vec ? row_norms_kernel<T, TPR, true> : row_norms_kernel<T, TPR, false>, grid, \
+                                 kThreads, 0, s, g, m, n, ldg, norms));                         \
   }
   GRASS_NORMS_CASE(32) GRASS_NORMS_CASE(64) GRASS_NORMS_CASE(128) GRASS_NORMS_CASE(256)
 #undef GRASS_NORMS_CASE
-  GRASS_LAUNCH_CHECK();
   return GRASS_OK;
 }
 

@@ -496,7 +496,7 @@ int allow_smem(K kernel, bool (&done)[64]) {
 }
 
 // Ranking: eight CTAs (the portable cluster size) from 4097 rows up, else one.
-int launch_rank(SelectArgs& a, cudaStream_t s, bool dependent) {
+int launch_rank(SelectArgs& a, cudaStream_t s) {
   const int ctas = a.m > 4 * kThreads ? 8 : 1;
   const int rows = static_cast<int>(round_up((static_cast<size_t>(a.m) + ctas - 1) / ctas, 32));
   a.stage_norms = rows * sizeof(float) <= kSelectBudget;
@@ -514,7 +514,7 @@ int launch_rank(SelectArgs& a, cudaStream_t s, bool dependent) {
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
   attr[1] = dependent_launch_attr();
   cfg.attrs = attr;
-  cfg.numAttrs = dependent ? 2 : 1;
+  cfg.numAttrs = 2;
   ProfileScope prof(GRASS_K_SELECT, s);
   GRASS_CUDA_TRY(cudaLaunchKernelEx(&cfg, select_rank_kernel, a, rows));
   return GRASS_OK;
@@ -523,8 +523,8 @@ int launch_rank(SelectArgs& a, cudaStream_t s, bool dependent) {
 // Stage the norms (and, if they still fit, the hit counters and the running sum) in shared memory: the
 // with-replacement kernel is a chain of short passes over m values, each of which would otherwise wait
 // on an L2 round trip.
-int launch_select(SelectArgs& a, cudaStream_t s, bool dependent) {
-  if (a.method == GRASS_SEL_TOPR || is_nr(a.method)) return launch_rank(a, s, dependent);
+int launch_select(SelectArgs& a, cudaStream_t s) {
+  if (a.method == GRASS_SEL_TOPR || is_nr(a.method)) return launch_rank(a, s);
   const size_t m4 = (static_cast<size_t>(a.m) + 3) / 4 * 4 * sizeof(float);
   a.stage_norms = m4 <= kSelectBudget;
   a.stage_counts = a.stage_norms && 2 * m4 <= kSelectBudget;
@@ -534,7 +534,7 @@ int launch_select(SelectArgs& a, cudaStream_t s, bool dependent) {
   const int rc = allow_smem(select_kernel, attr_set);
   if (rc != GRASS_OK) return rc;
   ProfileScope prof(GRASS_K_SELECT, s);
-  GRASS_CUDA_TRY(launch_kernel(select_kernel, 1, kThreads, smem, s, dependent, a));
+  GRASS_CUDA_TRY(launch_kernel(select_kernel, 1, kThreads, smem, s, a));
   return GRASS_OK;
 }
 
@@ -550,7 +550,7 @@ extern "C" size_t grass_select_workspace_bytes(int64_t m, int32_t r, int method)
   return grass::cdf_bytes(m) + grass::round_up(static_cast<size_t>(m) * sizeof(int), 256);
 }
 
-int grass::select_rows(bool dependent, const float* norms, int64_t m, int32_t r, int method, uint64_t seed,
+int grass::select_rows(const float* norms, int64_t m, int32_t r, int method, uint64_t seed,
                        uint32_t layer_id, uint32_t epoch, int32_t* idx, float* rho, void* ws,
                        size_t ws_bytes, cudaStream_t s) {
   if (norms == nullptr || idx == nullptr || rho == nullptr || m < 1 || m > 0x7fffffffLL ||
@@ -580,13 +580,13 @@ int grass::select_rows(bool dependent, const float* norms, int64_t m, int32_t r,
   a.epoch = epoch;
   a.idx = idx;
   a.rho = rho;
-  return launch_select(a, s, dependent);
+  return launch_select(a, s);
 }
 
 extern "C" int grass_select(const float* norms, int64_t m, int32_t r, int method, uint64_t seed,
                             uint32_t layer_id, uint32_t epoch, int32_t* idx, float* rho, void* ws,
                             size_t ws_bytes, void* stream) {
-  return grass::select_rows(false, norms, m, r, method, seed, layer_id, epoch, idx, rho, ws, ws_bytes,
+  return grass::select_rows(norms, m, r, method, seed, layer_id, epoch, idx, rho, ws, ws_bytes,
                             static_cast<cudaStream_t>(stream));
 }
 
@@ -659,5 +659,5 @@ extern "C" int grass_select_static(const float* norms, int64_t m, int32_t r, int
   // with-replacement method (everything else is staged in shared memory); it writes every
   // running-sum entry before reading it, so whatever an earlier call left there is never
   // observed.
-  return launch_select(a, static_cast<cudaStream_t>(stream), false);
+  return launch_select(a, static_cast<cudaStream_t>(stream));
 }

@@ -107,23 +107,23 @@ __device__ __forceinline__ float ld_f32(const float* p) {
   return v;
 }
 
-// 16-bit read-only load that does not allocate in L1 (each selected column is read once).  An L2
+// 16-bit load that does not allocate in L1 (each selected column is read once).  An L2
 // miss fetches 128 bytes by default; HALF_LINE lowers the prefetch size to 64 bytes, which is what
 // an isolated pick should pay for (16 M isolated 2-byte reads: 276 -> 165 us).
 template <bool HALF_LINE>
-__device__ __forceinline__ unsigned short ld_nc_na_u16(const unsigned short* p) {
+__device__ __forceinline__ unsigned short ld_na_u16(const unsigned short* p) {
   unsigned short v;
   if (HALF_LINE)
-    asm volatile("ld.global.nc.L1::no_allocate.L2::64B.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    asm volatile("ld.global.L1::no_allocate.L2::64B.u16 %0, [%1];" : "=h"(v) : "l"(p));
   else
-    asm volatile("ld.global.nc.L1::no_allocate.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    asm volatile("ld.global.L1::no_allocate.u16 %0, [%1];" : "=h"(v) : "l"(p));
   return v;
 }
 
 // The same, allocating in L1 (neighbouring lanes of other warps read the same lines).
-__device__ __forceinline__ unsigned short ld_nc_u16(const unsigned short* p) {
+__device__ __forceinline__ unsigned short ld_u16(const unsigned short* p) {
   unsigned short v;
-  asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(v) : "l"(p));
+  asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
   return v;
 }
 

@@ -293,3 +293,64 @@ def test_the_separate_gather_copies_what_the_cooperative_one_does(T, r, m):
     grass.grass_device_status()
     want = dY[:, idx.long()].double().T @ X.double()
     assert torch.equal(*out) and rel(out[0], want) <= 1e-5
+
+
+@pytest.mark.parametrize("shape", [(2048, 512, 512, 128), (2048, 1024, 512, 256), (4096, 512, 256, 128)])
+@pytest.mark.parametrize("gather", [grass.binding.GATHER_AUTO, grass.binding.GATHER_PREPASS,
+                                    grass.binding.GATHER_COOPERATIVE, grass.binding.GATHER_IN_CTA])
+def test_a_projection_waits_for_the_kernel_that_makes_its_inputs(shape, gather):
+    """The first kernel of a call is placed while the program's kernel before it drains: what that one writes (here new
+    dY and X on every iteration, right before the call) is what the projection reads, eagerly and in a graph
+    that forks and joins streams before the call."""
+    T, m, n, r = shape
+    r = 64 if gather == grass.binding.GATHER_IN_CTA else r
+    base_dY, base_X, _ = inputs(T, m, n)
+    dY, X = torch.zeros_like(base_dY), torch.zeros_like(base_X)
+    idx, opts = rows_of(m, r), dict(gather=gather)
+    ws = torch.empty(grass.grass_project_plan(1, T, m, n, r, opts)["workspace_bytes"], dtype=torch.uint8, device=DEV)
+    Gc, want = torch.empty((r, n), device=DEV), torch.empty((r, n), device=DEV)
+
+    def project(a, b, out):
+        grass.binding.grass_project_grad_ex([a], [b], [idx], [None], r, [out], ws, opts)
+
+    project(base_dY, base_X, want)
+    seen = []
+    for k in range(30):                                    # powers of two: exact in bf16 and fp32
+        torch.mul(base_dY, 2.0 ** (k % 5), out=dY)
+        torch.mul(base_X, 2.0 ** -(k % 3), out=X)
+        project(dY, X, Gc)
+        seen.append((Gc.clone(), 2.0 ** (k % 5 - k % 3)))
+    for got, scale in seen:
+        assert torch.equal(got, want * scale)
+    main, side = torch.cuda.Stream(), torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=main):
+        side.wait_stream(main)
+        with torch.cuda.stream(side):
+            dY.copy_(base_dY)
+        X.zero_()
+        X.add_(base_X)
+        main.wait_stream(side)
+        project(dY, X, Gc)
+        dY.mul_(2.0)
+        project(dY, X, Gc)
+    for _ in range(3):
+        Gc.zero_()
+        dY.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(Gc, want * 2.0)
+    grass.grass_device_status()
+
+
+def test_row_norms_and_selection_wait_for_the_kernel_before():
+    G, norms = torch.empty((3000, 700), device=DEV), torch.empty(3000, device=DEV)
+    idx, rho = torch.zeros(64, dtype=torch.int32, device=DEV), torch.zeros(64, device=DEV)
+    for k in range(20):
+        G.fill_(0.0)
+        G[k:k + 64] = 2.0 ** k
+        grass.grass_row_norms(G, norms)
+        grass.grass_select(norms, 64, grass.SEL_TOPR, 0, 0, 0, idx, rho, None)
+        assert torch.equal(idx.long(), torch.arange(k, k + 64, device=DEV))
+    grass.grass_device_status()
