@@ -770,12 +770,11 @@ TcPlan make_norms_plan(int64_t T, int64_t m, int64_t n, bool* small = nullptr) {
   return make_plan(T, m, n, static_cast<int>(m), false, o, !few_tiles);
 }
 
-// A refresh whose small dense gradient also serves as G_C: where it leaves the partials.
+// A refresh whose small dense gradient also serves as G_C: where the norms leave it, its partials summed.
 struct GradParts {
   int r = 0;                       // in: rows that will be selected
-  const float* part = nullptr;     // out
-  long long ld = 0, stride = 0;
-  int split_k = 0;                 // 0: the gradient was not kept
+  const float* grad = nullptr;     // out; NULL: not kept
+  long long ld = 0;
 };
 size_t grad_parts_bytes(int split_k, int64_t m, long long ld) {
   return round_up(static_cast<size_t>(split_k) * m * ld * sizeof(float), 256);
@@ -834,12 +833,14 @@ int plan_refused(const TcPlan& plan, int64_t T, size_t need, const void* ws, siz
 
 // Rows of up to 128, 256 and 512 columns (four a thread) share a CTA, as long as two CTAs an SM are left (256 rows
 // of 256 columns in 16 splits, an fp32 refresh step: 21.6 us with a CTA each, 22.8 with four a CTA).
-cudaError_t launch_row_norms(const float* part, long long ld, long long stride, int split_k, int64_t m, int64_t n,
-                             float* norms, cudaStream_t s) {
+cudaError_t launch_row_norms(float* part, long long ld, long long stride, int split_k, int64_t m, int64_t n,
+                             float* norms, bool keep, cudaStream_t s) {
   int threads = n <= 128 ? 32 : n <= 256 ? 64 : n <= 512 ? 128 : 256;
   while (threads < 256 && m * threads / 256 < 2 * kSmCount) threads *= 2;
   const int rows = 256 / threads;
-  auto kernel = threads < 256 ? splitk_rownorms_kernel<true> : splitk_rownorms_kernel<false>;
+  keep = keep && split_k > 1;               // (one partial is the sum)
+  auto kernel = threads < 256 ? keep ? splitk_rownorms_kernel<true, true> : splitk_rownorms_kernel<true, false>
+                              : keep ? splitk_rownorms_kernel<false, true> : splitk_rownorms_kernel<false, false>;
   return launch_kernel(kernel, static_cast<unsigned>((m + rows - 1) / rows), 256, 0, s, part, ld, stride,
                        split_k, static_cast<int>(m), static_cast<int>(n), threads, norms);
 }
@@ -991,8 +992,8 @@ int project_bf16(int count, const void* const* dY, int64_t lddy, const void* con
                                    p.norm_part, p.ld_norm, static_cast<int>((n + 31) / 32),
                                    static_cast<int>(m), norms));
     else
-      GRASS_CUDA_TRY(launch_row_norms(part[0], plan.ld_part, p.split_stride, plan.split_k, m, n, norms, s));
-    if (stored) *keep = {keep->r, part[0], plan.ld_part, p.split_stride, plan.split_k};
+      GRASS_CUDA_TRY(launch_row_norms(part[0], plan.ld_part, p.split_stride, plan.split_k, m, n, norms, stored, s));
+    if (stored) *keep = {keep->r, part[0], plan.ld_part};
     return GRASS_OK;
   }
   if (upd != nullptr) {
@@ -1094,8 +1095,8 @@ int project_fp32(const void* dY, int64_t lddy, const void* X, int64_t ldx, int64
     // row-norm mode (idx NULL, r == m): the norms straight from the partials
     ProfileScope prof(GRASS_K_ROW_NORMS, s);
     const long long stride = static_cast<long long>(r) * fp.ld_part;
-    GRASS_CUDA_TRY(launch_row_norms(out, ld_out, stride, fp.split, m, n, norms, s));
-    if (keep != nullptr) *keep = {keep->r, out, static_cast<long long>(ld_out), stride, fp.split};
+    GRASS_CUDA_TRY(launch_row_norms(out, ld_out, stride, fp.split, m, n, norms, keep != nullptr, s));
+    if (keep != nullptr) *keep = {keep->r, out, static_cast<long long>(ld_out)};
     return GRASS_OK;
   }
   if (upd != nullptr) {
@@ -1320,11 +1321,10 @@ extern "C" int grass_refresh_step(const grass_step_t* a, const grass_refresh_t* 
                      f->select_ws_bytes, s);
   if (rc2 != GRASS_OK) return rc2;
   u.reset = f->reset_state != 0;
-  if (kept.split_k == 0) return project_and_update(a, u, s, true);
-  u.grp.part[0] = kept.part;
+  if (kept.grad == nullptr) return project_and_update(a, u, s, true);
+  u.grp.part[0] = kept.grad;
   u.ld_part = kept.ld;
-  u.split_stride = kept.stride;
-  u.split_k = kept.split_k;
+  u.split_k = 1;
   u.part_by_row = true;
   return launch_update(u, s);
 }

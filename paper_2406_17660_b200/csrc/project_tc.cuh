@@ -920,10 +920,12 @@ splitk_reduce_kernel(const ReduceGroup grp, long long ld_part, long long split_s
 // a shuffle tree and one shared-memory hop: bit-reproducible, whatever row_threads is.
 // Bound by the latency of its loads where rows are short, so no thread is left without any (5461 rows of 91
 // columns in 13 splits: 37 us with a CTA per row).
+// KEEP: the sums are left in the place of the first partial, for the update that takes its rows from there: 4 m n bytes
+// more here, and 1 partial instead of split_k to read there, in the same order of adds.
 // SHORT: row_threads as given (32, 64 or 128); else 256, known to the compiler.
-template <bool SHORT>
+template <bool SHORT, bool KEEP>
 __global__ void __launch_bounds__(256)
-splitk_rownorms_kernel(const float* part, long long ld_part, long long split_stride,
+splitk_rownorms_kernel(float* part, long long ld_part, long long split_stride,
                        int split_k, int m, int n, int short_row_threads, float* norms) {
   __shared__ float s_part[8];
   grid_dep_launch();
@@ -931,10 +933,10 @@ splitk_rownorms_kernel(const float* part, long long ld_part, long long split_str
   const int row_threads = SHORT ? short_row_threads : 256;
   const int warp = threadIdx.x >> 5, t = threadIdx.x & (row_threads - 1);
   const int j = blockIdx.x * (256 / row_threads) + threadIdx.x / row_threads;
-  const float* row = part + static_cast<long long>(j) * ld_part;
+  float* row = part + static_cast<long long>(j) * ld_part;
   float acc = 0.f;
   for (int c = j < m ? 4 * t : n; c < n; c += 4 * row_threads) {
-    const float* p = row + c;
+    float* p = row + c;
     float4 g = *reinterpret_cast<const float4*>(p);
     for (int s = 1; s < split_k; s += 4) {
       float4 t[4];
@@ -948,6 +950,7 @@ splitk_rownorms_kernel(const float* part, long long ld_part, long long split_str
         g.x += t[u].x; g.y += t[u].y; g.z += t[u].z; g.w += t[u].w;
       }
     }
+    if (KEEP) *reinterpret_cast<float4*>(p) = g;
     acc = fmaf(g.x, g.x, acc);
     if (c + 1 < n) acc = fmaf(g.y, g.y, acc);
     if (c + 2 < n) acc = fmaf(g.z, g.z, acc);
