@@ -10,7 +10,9 @@
 // Ranking (Top-r and without replacement) costs every row a score and six looks, so it runs on a
 // cluster of eight CTAs, about two rows a thread, that exchange histograms and counts through
 // distributed shared memory: 13824 rows without replacement took 37 us on one CTA, 14 on eight; up to
-// 4096 rows one CTA is as fast (10 us at 4096, 12 on a cluster: six cluster barriers).
+// 4096 rows one CTA is as fast for Top-r (10 us at 4096, 12 on a cluster: six cluster barriers).  A score costs a Philox
+// block and an fp64 logarithm, so without replacement the cluster pays from 1025 rows (9.6 us either way there; 2368 rows
+// 11.3 -> 9.6, 4096 rows 13.6 -> 9.7).
 // Sampling with replacement is a serial chain (running sum, search, expansion) and stays on one.
 //
 //   Top-r: the fp32 bit pattern of a non-negative float orders like the float,
@@ -495,9 +497,9 @@ int allow_smem(K kernel, bool (&done)[64]) {
   return GRASS_OK;
 }
 
-// Ranking: eight CTAs (the portable cluster size) from 4097 rows up, else one.
+// Ranking: eight CTAs (the portable cluster size) from 4097 rows up, 1025 where rows are scored, else one.
 int launch_rank(SelectArgs& a, cudaStream_t s) {
-  const int ctas = a.m > 4 * kThreads ? 8 : 1;
+  const int ctas = a.m > (is_nr(a.method) ? 1 : 4) * kThreads ? 8 : 1;
   const int rows = static_cast<int>(round_up((static_cast<size_t>(a.m) + ctas - 1) / ctas, 32));
   a.stage_norms = rows * sizeof(float) <= kSelectBudget;
   static bool attr_set[64] = {false};
