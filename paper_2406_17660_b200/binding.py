@@ -578,7 +578,7 @@ class LayerStepCall:
             raise TypeError("a layer step takes CUDA tensors")
         now = (dY.shape, X.shape, dY.stride(), X.stride(), dY.dtype, X.dtype)
         if g == 0:
-            yshape, xshape, ystride, xstride, dt, dt2 = self._now = now
+            yshape, xshape, ystride, xstride, dt, dt2 = now
             if len(yshape) != 2 or len(xshape) != 2:
                 raise ValueError("expected a 2-D tensor with unit inner stride")
             if yshape[0] != xshape[0] or dt is not dt2:
@@ -594,7 +594,7 @@ class LayerStepCall:
             a, T = self.args, xshape[0]
             a.T, a.dt = T, code
             a.lddy, a.ldx = (ystride[0], xstride[0]) if T > 1 else (max(ystride[0], m), max(xstride[0], n))
-            self._alike_inputs = seen
+            self._now, self._alike_inputs = now, seen     # one record: a refused pair leaves neither
         elif now != self._now and not (             # (one token has no pitch)
                 now[0][0] == 1 and now[:2] == self._now[:2] and now[4:] == self._now[4:]
                 and now[2][1] == now[3][1] == 1):

@@ -345,3 +345,48 @@ def test_a_scanned_call_is_checked_again_when_layer_0_changes(calls, monkeypatch
         call.inputs(0, torch.zeros(T, M, dtype=torch.bfloat16), torch.zeros(T, N, dtype=torch.bfloat16))
     with pytest.raises(ValueError):
         call.state(0, **plain, cols=True)
+
+
+@pytest.fixture
+def plain(calls, monkeypatch):
+    """Tensors that the scan takes (it leaves subclasses to the checks) and that pass for CUDA tensors."""
+    monkeypatch.setattr(torch.Tensor, "is_cuda", True)
+
+    def plain_group(count=2, tokens=16):
+        layers = [layer(t=1, K=1 << 30, tokens=tokens) for _ in range(count)]
+        for l in layers:
+            for name in ("W", "idx", "rho", "Gc", "M", "V", "U"):
+                setattr(l, name, getattr(l, name).as_subclass(torch.Tensor))
+        return grass.step.GrassLayerGroup(layers, tokens, device="cpu")
+
+    return plain_group
+
+
+def zeros(*shapes):
+    return [torch.zeros(shape, dtype=torch.bfloat16) for shape in shapes]
+
+
+@pytest.mark.parametrize("bad", [((4, M), (16, N)), ((16, M), (15, N)), ((16, M - 1), (16, N))],
+                         ids=["few of dY", "few of X", "narrow"])
+def test_inputs_go_with_the_ones_that_layer_0_was_let_through_with(calls, plain, bad):
+    """Not with those that it was refused with: what goes with them would be read past its end."""
+    group, good = plain(), zeros((16, M), (16, N))
+    group.step([good[0]] * 2, [good[1]] * 2)
+    refused = zeros(*bad)
+    for g in range(2):                                   # as layer 0's, then as layer 1's
+        pairs = [refused, good] if g == 0 else [good, refused]
+        with pytest.raises(ValueError):
+            group.step(*map(list, zip(*pairs)))
+    assert len(calls) == 1
+    group.step([good[0], gpu(16, M, dtype=torch.bfloat16)], [good[1], gpu(16, N, dtype=torch.bfloat16)])
+    assert calls[-1][1]["T"] == 16 and len(calls) == 2
+
+
+def test_a_single_token_of_another_pitch_goes_with_layer_0_after_a_refusal(calls, plain):
+    group = plain()
+    wide = zeros((4, M + 16))[0][:1, :M]
+    group.step([zeros((1, M))[0], wide], zeros((1, N), (1, N)))
+    with pytest.raises(ValueError):
+        group.step(zeros((2, M), (1, M)), zeros((3, N), (1, N)))
+    group.step([zeros((1, M))[0], wide], zeros((1, N), (1, N)))
+    assert calls[-1][1]["dY"][1] == wide.data_ptr() and calls[-1][1]["T"] == 1
