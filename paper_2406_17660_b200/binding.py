@@ -543,6 +543,7 @@ class LayerStepCall:
             raise TypeError(f"unsupported dtype {W.dtype}")
         own = (r, n, wshape[k], code, ldm if Gc.stride() == stride else _ld(Gc), ldm, ldw, k)
         if g == 0:
+            self._forget()                 # the other layers and the inputs are compared with layer 0
             a = self.args
             self._own = own
             a.r, a.n, a.m, a.wdt, a.ldgc, a.ldstate, a.ldw, a.side = own
@@ -553,8 +554,6 @@ class LayerStepCall:
         sr[g] = None if rho is None else rho.data_ptr()
         sg[g], sm[g], sv[g], sw[g] = Gc.data_ptr(), M.data_ptr(), V.data_ptr(), W.data_ptr()
         su[g] = None if U is None else U.data_ptr()
-        if g == 0:
-            self._forget()                 # the other layers and the inputs are compared with layer 0
         self._alike[k][g] = seen
 
     def layers_are(self, owns):

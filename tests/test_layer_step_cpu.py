@@ -390,3 +390,18 @@ def test_a_single_token_of_another_pitch_goes_with_layer_0_after_a_refusal(calls
         group.step(zeros((2, M), (1, M)), zeros((3, N), (1, N)))
     group.step([zeros((1, M))[0], wide], zeros((1, N), (1, N)))
     assert calls[-1][1]["dY"][1] == wide.data_ptr() and calls[-1][1]["T"] == 1
+
+
+def test_a_layer_0_that_has_no_address_leaves_nothing_of_itself(calls, plain):
+    """Its sizes are in the call by then: the layer 0 before it is checked, and put in, again."""
+    class Nowhere(OnGpu):
+        def data_ptr(self):
+            raise RuntimeError("no storage")
+
+    good = {k: torch.zeros(v.shape, dtype=v.dtype) for k, v in buffers().items()}
+    call = B.LayerStepCall()
+    call.state(0, **good)
+    with pytest.raises(RuntimeError):
+        call.state(0, **dict(buffers(r=R - 1), M=torch.zeros(R - 1, N).as_subclass(Nowhere)))
+    call.state(0, **good)
+    assert call.args.r == R and call.args.M[0] == good["M"].data_ptr()
