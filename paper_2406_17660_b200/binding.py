@@ -462,7 +462,6 @@ def grass_refresh_keeps_gradient(T: int, m: int, n: int, r: int, dt: int) -> boo
     return bool(load_library().grass_refresh_keeps_gradient(T, m, n, r, dt))
 
 
-_data_ptr = torch.Tensor.data_ptr
 _F32, _I32 = torch.float32, torch.int32
 _CODES = {torch.float32: F32, torch.bfloat16: BF16}
 
@@ -497,7 +496,7 @@ class LayerStepCall:
         self._refresh_ref = ctypes.byref(f)
         lib = load_library()
         self._launch, self._launch_refresh = lib.grass_layer_step, lib.grass_refresh_step
-        self._now = self._held = self._pointers = None
+        self._now = None
         self._accepted = _accepted()
         self._at = ctypes.addressof(a) + LayerStep.dY.offset     # of the pointers: nine fields of MAX_GROUP each
         self._forget()
@@ -555,18 +554,6 @@ class LayerStepCall:
         sg[g], sm[g], sv[g], sw[g] = Gc.data_ptr(), M.data_ptr(), V.data_ptr(), W.data_ptr()
         su[g] = None if U is None else U.data_ptr()
         self._alike[k][g] = seen
-
-    def layers_are(self, owns):
-        """Whether the tensors that state() was given (all layers', as in the last layers_were()) lie where they
-        lay then; if not, state() is due for every layer.  A group asks on every step, since state() takes
-        2.8 us a layer and this 0.5.  The tensors are held: no other can come to lie at the address of one."""
-        if list(map(_data_ptr, owns)) == self._pointers:
-            return True
-        self._pointers = None
-        return False
-
-    def layers_were(self, owns):
-        self._held, self._pointers = owns, list(map(_data_ptr, owns))
 
     def inputs(self, g, dY, X):
         """Layer g's dY (T x m) and X (T x n); after state(0, ..)."""

@@ -153,16 +153,9 @@ class GrassLayerGroup:
 
     def _marshal(self):
         """The buffers that the layers have now: a layer may have been given others since the last step."""
-        owns = []
-        for l in self.layers:
-            owns += l.idx, l.rho, l.Gc, l.M, l.V, l.W
-            if l.keep_U:
-                owns.append(l.U)
-        call = self._call
-        if not call.layers_are(owns):
-            for g, l in enumerate(self.layers):
-                call.state(g, l.idx, l.rho, l.Gc, l.M, l.V, l.U if l.keep_U else None, l.W)
-            call.layers_were(owns)
+        state = self._call.state
+        for g, l in enumerate(self.layers):
+            state(g, l.idx, l.rho, l.Gc, l.M, l.V, l.U if l.keep_U else None, l.W)
 
     def step(self, dYs, Xs):
         ls = self.layers

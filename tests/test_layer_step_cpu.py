@@ -405,3 +405,20 @@ def test_a_layer_0_that_has_no_address_leaves_nothing_of_itself(calls, plain):
         call.state(0, **dict(buffers(r=R - 1), M=torch.zeros(R - 1, N).as_subclass(Nowhere)))
     call.state(0, **good)
     assert call.args.r == R and call.args.M[0] == good["M"].data_ptr()
+
+
+@pytest.mark.parametrize("name,view", [("W", lambda t: t.view(torch.float16)), ("V", lambda t: t[:R - 1]),
+                                       ("M", lambda t: t.view(R // 2, 2 * N)), ("idx", lambda t: t[:R - 1]),
+                                       ("Gc", lambda t: t.view(torch.int32))], ids=["W", "V", "M", "idx", "Gc"])
+def test_a_groups_buffer_of_another_form_at_the_same_address_is_refused(calls, plain, name, view):
+    group = plain()
+    inputs = zeros((16, M), (16, M)), zeros((16, N), (16, N))
+    group.step(*inputs)
+    held, l = getattr(group.layers[1], name), group.layers[1]
+    setattr(l, name, view(held))
+    assert getattr(l, name).data_ptr() == held.data_ptr()
+    with pytest.raises((TypeError, ValueError)):
+        group.step(*inputs)
+    setattr(l, name, held)
+    group.step(*inputs)
+    assert len(calls) == 2
