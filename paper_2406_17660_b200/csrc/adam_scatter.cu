@@ -15,10 +15,6 @@
 // one contiguous run of 128 bytes: the r = 512, n = 5461 update takes 20 us cold; eight consecutive
 // scalars a thread took 49.
 //
-// As a dependent launch after the projection of a regular iteration (`early`) a block reads idx, rho, M, V and W, which
-// are inputs of the call, before it waits for the kernel that writes the gradient: their latency then passes while that
-// kernel drains (60M q, T = 2048: a step 11.5 -> 10.8 us; 13B down, T = 4096: 176.9 -> 170.0).
-//
 // idx is ascending, so repeated rows are adjacent (a "run"; sampling with replacement gives runs of
 // two to hundreds).  The W row is rounded once, after the terms of its run are added in order of
 // j.  A run costs a few memory latencies a row when one warp walks it, so longer runs are taken by
@@ -99,7 +95,7 @@ struct RowArgs {
   int64_t ldgc, ldstate, n;
   long long ld_part, split_stride;
   int split_k;
-  bool part_by_row, reset, early;
+  bool part_by_row, reset;
 };
 
 // Gradient (the partials' sum, or Gc itself) and Adam of row j at this lane's columns; `row` is
@@ -116,7 +112,6 @@ __device__ __forceinline__ void update_row(const RowArgs& p, const AdamScalars& 
     load_e<E, VEC>(mrow, c, p.n, mv);
     load_e<E, VEC>(vrow, c, p.n, vv);
   }
-  if (p.early) grid_dep_wait();
   if (SPLIT) {
     const int pr = p.part_by_row ? row : j;
     if (pr < 0) rho = 0.f;
@@ -159,15 +154,15 @@ __global__ void __launch_bounds__(kThreads, SPLIT ? 4 : 6)
 adam_apply_narrow_kernel(const __grid_constant__ UpdateGroup grp, int64_t ldgc, int64_t ldstate,
                          int64_t m, int64_t n, int64_t ldw, int r, long long ld_part,
                          long long split_stride, int split_k, bool part_by_row, bool reset,
-                         bool early, float alpha, AdamScalars a, int* status) {
+                         float alpha, AdamScalars a, int* status) {
   __shared__ float s_u[kRows][32];
   __shared__ float s_scale[kRows];
-  if (!early) grid_dep_wait();
+  grid_dep_wait();
   const int lay = blockIdx.z;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int32_t* idx = grp.idx[lay];
   const RowArgs p = {grp.part[lay], grp.Gc[lay], grp.M[lay], grp.V[lay], grp.U[lay], grp.rho[lay],
-                     ldgc, ldstate, n, ld_part, split_stride, split_k, part_by_row, reset, early};
+                     ldgc, ldstate, n, ld_part, split_stride, split_k, part_by_row, reset};
   const int64_t c = static_cast<int64_t>(blockIdx.x) * 32 + lane;
   const int ja = blockIdx.y * kRows, j = ja + warp;
   const int last = ja + kRows < r ? ja + kRows : r;       // rows of this block: [ja, last)
@@ -270,15 +265,14 @@ template <typename T, int E, bool VEC, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 4)
 adam_apply_wide_kernel(const __grid_constant__ UpdateGroup grp, int64_t ldgc, int64_t ldstate, int64_t m,
                        int64_t n, int64_t ldw, int r, long long ld_part, long long split_stride,
-                       int split_k, bool part_by_row, bool reset, bool early, float alpha, AdamScalars a,
-                       int* status) {
+                       int split_k, bool part_by_row, bool reset, float alpha, AdamScalars a, int* status) {
   __shared__ float s_u[kThreads / 32][128];               // long runs only
   __shared__ float s_scale[kThreads / 32];
-  if (!early) grid_dep_wait();
+  grid_dep_wait();
   const int lay = blockIdx.z, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int32_t* idx = grp.idx[lay];
   const RowArgs p = {grp.part[lay], grp.Gc[lay], grp.M[lay], grp.V[lay], grp.U[lay], grp.rho[lay],
-                     ldgc, ldstate, n, ld_part, split_stride, split_k, part_by_row, reset, early};
+                     ldgc, ldstate, n, ld_part, split_stride, split_k, part_by_row, reset};
   const int j0 = blockIdx.y;
   const int row = idx[j0];
   const bool prev = j0 > 0 && idx[j0 - 1] == row, next = j0 + 1 < r && idx[j0 + 1] == row;
@@ -338,11 +332,10 @@ template <typename T, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 4)
 adam_apply_cols_kernel(const __grid_constant__ UpdateGroup grp, int64_t ldgc, int64_t ldstate, int64_t m,
                        int64_t n, int64_t ldw, int r, long long ld_part, long long split_stride,
-                       int split_k, bool part_by_row, bool reset, bool early, float alpha, AdamScalars a,
-                       int* status) {
+                       int split_k, bool part_by_row, bool reset, float alpha, AdamScalars a, int* status) {
   constexpr int J = 32, Q = 4;                            // state rows of a block, of a warp
   __shared__ float s_u[J][33];
-  if (!early) grid_dep_wait();
+  grid_dep_wait();
   const int lay = blockIdx.z, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int32_t* idx = grp.idx[lay];
   const float* rho = grp.rho[lay];
@@ -383,15 +376,6 @@ adam_apply_cols_kernel(const __grid_constant__ UpdateGroup grp, int64_t ldgc, in
       const int js = on[q] ? j : base;
       rj[q] = rho != nullptr ? rho[js] : 1.f;
       s[q] = alpha * rj[q];
-      if (on[q] && !reset) {
-        mv[q] = M[static_cast<int64_t>(j) * ldstate + c];
-        vv[q] = V[static_cast<int64_t>(j) * ldstate + c];
-      }
-    }
-    if (early) grid_dep_wait();
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      const int j = base + Q * warp + q, js = on[q] ? j : base;
       if (SPLIT) {
         int pr = js;
         if (part_by_row) {
@@ -402,6 +386,10 @@ adam_apply_cols_kernel(const __grid_constant__ UpdateGroup grp, int64_t ldgc, in
         g[q] = *p[q];
       } else if (on[q]) {
         g[q] = Gc[j * ldgc + c];
+      }
+      if (on[q] && !reset) {
+        mv[q] = M[static_cast<int64_t>(j) * ldstate + c];
+        vv[q] = V[static_cast<int64_t>(j) * ldstate + c];
       }
     }
     if (SPLIT) {
@@ -474,7 +462,7 @@ int launch_cols(const UpdateCall& u, cudaStream_t s) {
   ProfileScope prof(GRASS_K_ADAM_SCATTER, s);
   GRASS_CUDA_TRY(launch_kernel(u.split_k > 0 ? adam_apply_cols_kernel<T, true> : adam_apply_cols_kernel<T, false>,
                                grid, kThreads, 0, s, u.grp, u.ldgc, u.ldstate, u.m, u.n, u.ldw,
-                               u.r, u.ld_part, u.split_stride, u.split_k, u.part_by_row, u.reset, u.early, u.alpha,
+                               u.r, u.ld_part, u.split_stride, u.split_k, u.part_by_row, u.reset, u.alpha,
                                u.a, status));
   return GRASS_OK;
 }
@@ -487,7 +475,7 @@ int launch_narrow(const UpdateCall& u, int* status, cudaStream_t s) {
     ProfileScope prof(GRASS_K_ADAM_SCATTER, s);
     GRASS_CUDA_TRY(launch_kernel(adam_apply_narrow_kernel<T, SPLIT>, grid, kThreads, 0, s,
         u.grp, u.ldgc, u.ldstate, u.m, u.n, u.ldw, u.r, u.ld_part, u.split_stride, u.split_k, u.part_by_row,
-        u.reset, u.early, u.alpha, u.a, status));
+        u.reset, u.alpha, u.a, status));
   }
   return GRASS_OK;
 }
@@ -510,7 +498,7 @@ int launch_wide(const UpdateCall& u, int* status, cudaStream_t s) {
     GRASS_CUDA_TRY(launch_kernel(
         vec ? adam_apply_wide_kernel<T, E, true, SPLIT> : adam_apply_wide_kernel<T, E, false, SPLIT>, grid,
         threads, 0, s, u.grp, u.ldgc, u.ldstate, u.m, u.n, u.ldw, u.r, u.ld_part,
-        u.split_stride, u.split_k, u.part_by_row, u.reset, u.early, u.alpha, u.a, status));
+        u.split_stride, u.split_k, u.part_by_row, u.reset, u.alpha, u.a, status));
   }
   return GRASS_OK;
 }

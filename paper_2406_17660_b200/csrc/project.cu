@@ -1220,7 +1220,6 @@ int check_step(const grass_step_t* a, UpdateCall& u) {
 // refresh: the projection of a refresh iteration, with the token slices of the projection calls
 // (make_keep_plan says why).
 int project_and_update(const grass_step_t* a, UpdateCall& u, cudaStream_t s, bool refresh = false) {
-  u.early = !refresh;                  // (a refresh's selection writes idx and rho in the same call)
   if (a->dt == GRASS_F32)
     return project_fp32(a->dY[0], a->lddy, a->X[0], a->ldx, a->T, a->m, a->n, a->idx[0], a->rho[0],
                         a->r, a->Gc[0], a->ldgc, a->ws, a->ws_bytes, s, &u, nullptr, nullptr,

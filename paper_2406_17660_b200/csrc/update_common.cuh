@@ -67,8 +67,6 @@ struct UpdateCall {
   long long ld_part, split_stride;
   int split_k;
   bool part_by_row, reset;
-  bool early;               // follows a kernel of the same call that writes only the gradient and that has itself waited
-                            // for what came before: all else may be read before that one has finished
   float alpha;
   AdamScalars a;
 };

@@ -354,3 +354,60 @@ def test_row_norms_and_selection_wait_for_the_kernel_before():
         grass.grass_select(norms, 64, grass.SEL_TOPR, 0, 0, 0, idx, rho, None)
         assert torch.equal(idx.long(), torch.arange(k, k + 64, device=DEV))
     grass.grass_device_status()
+
+
+@pytest.mark.parametrize("T,m,n,r,side,gather", [
+    (2048, 512, 512, 128, "rows", grass.GATHER_PREPASS), (4096, 512, 256, 64, "rows", grass.GATHER_IN_CTA),
+    (1024, 1024, 2736, 256, "rows", grass.GATHER_PREPASS), (6000, 4096, 5461, 1024, "rows", grass.GATHER_COOPERATIVE),
+    (2048, 1376, 512, 128, "cols", None), (512, 256, 256, 32, "rows", None),
+], ids=["narrow", "narrow in-CTA", "wide", "wide cooperative", "cols", "fp32"])
+def test_a_step_waits_for_the_kernels_that_write_its_state(T, m, n, r, side, gather):
+    """A program may write rows, scales, state and weights right before a regular step (a checkpoint loaded, rows of its
+    own): the update is that of what it wrote last, whichever of them that is, eagerly and in a graph."""
+    dtype = torch.float32 if T == 512 else BF16
+    if gather is not None:
+        assert grass.grass_step_plan(1, T, m, n, r)["gather"] == gather
+    dY, X, W = inputs(T, m, n, dtype=dtype)
+    rows, contract = (n, m) if side == "cols" else (m, n)
+    ws = grass.step.GrassWorkspace([(rows, contract)], T, r, dtype, grass.SEL_TOPR)
+    l = grass.GrassLayer(W, r, grass.SEL_TOPR, 1 << 30, 0.25, 1e-3, workspace=ws, side=side)
+    g = torch.Generator(device=DEV).manual_seed(r)
+    names = ("idx", "rho", "M", "V", "W")
+
+    def written(seed):
+        rho, V = (torch.rand(s, device=DEV, generator=g) + 0.5 for s in (r, (r, contract)))
+        return dict(idx=rows_of(rows, r, seed), rho=rho, V=V, M=torch.randn((r, contract), device=DEV, generator=g),
+                    W=(W.float() * (seed + 1)).to(dtype))
+
+    def step(put, last=0):
+        for k in names[last:] + names[:last]:
+            torch.mul(put[k], 1, out=getattr(l, k))          # (a kernel, where copy_ may be a copy)
+        l.t, l.adam_step = 1, 3
+        l.step(dY, X)
+
+    states, want = [written(0), written(1)], []
+    for put in states:
+        for k in names:
+            getattr(l, k).copy_(put[k])
+        torch.cuda.synchronize()
+        l.t, l.adam_step = 1, 3
+        l.step(dY, X)
+        torch.cuda.synchronize()
+        want.append([getattr(l, k).clone() for k in ("Gc", "M", "V", "U", "W")])
+    assert not torch.equal(want[0][4], want[1][4])
+    seen = []
+    for k in range(20):
+        step(states[k % 2], k // 2 % len(names))
+        seen.append([getattr(l, k).clone() for k in ("Gc", "M", "V", "U", "W")])
+    for k, got in enumerate(seen):
+        assert all(torch.equal(a, b) for a, b in zip(got, want[k % 2])), k
+    graph, stream = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=stream):
+        for k in range(2 * len(names) + 1):
+            step(states[k % 2], k // 2 % len(names))
+    for _ in range(3):
+        graph.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(getattr(l, k), b) for k, b in zip(("Gc", "M", "V", "U", "W"), want[0]))
+    grass.grass_device_status()
