@@ -791,8 +791,11 @@ struct GatherGroup {
 // A warp owns TU tokens at a time and 32 NI consecutive j: lane l loads j = jb + 32 i + l for i < NI, so one
 // load instruction covers 32 neighbouring selected columns (ascending idx: as few 32-byte sectors as the
 // selection allows) and one store instruction writes 64 contiguous bytes of Ag.  Bound by HBM where rows are long and by
-// loads in flight where they are short: a lane has 16 of them out at r_pad >= 128, whatever NI is, unconditionally
-// (clamped, the value discarded at the store: under a per-lane condition the warp would wait for each).  One token at a
+// loads in flight where they are short: a lane has 16 of them out, or 8 where NI is 2 (a warp has four tokens in all) and 2 a
+// live group of 32 in the last block of a width past 256.  They are unconditional (under a per-lane condition the warp
+// would wait for each) and the values of lanes past r are discarded at the store.  Those lanes load column 0, a line more a
+// token; at NI = 2, where a line counts, the first column of their group, which is fetched anyway (T = 65536, r = 48 of 5461,
+// n = 256: 53.4 -> 52.2 us; from r = 65 up between 1 % faster and 1 % slower).  One token at a
 // time, 4 loads at r = 128, a step took 65.7 us where it takes 57.3 now (T = 65536, 512 x 1376); 29.2 and 25.6
 // (T = 22790, 359 x 1024).
 template <int NI, bool SPARSE>
@@ -806,7 +809,7 @@ gather_cols_kernel(const GatherGroup grp, long long lddy, int T, int m, int r, i
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int jb = blockIdx.x * (32 * NI);
   const int live = (r - jb + 31) / 32;      // groups of 32 columns that hold any
-  int rows[NI];
+  int rows[NI], from[NI];
 #pragma unroll
   for (int i = 0; i < NI; ++i) {
     const int j = jb + 32 * i + lane;
@@ -818,7 +821,11 @@ gather_cols_kernel(const GatherGroup grp, long long lddy, int T, int m, int r, i
         row = -1;
       }
     }
-    rows[i] = row;
+    rows[i] = from[i] = row;
+    if (NI == 2) {
+      const int first = __shfl_sync(0xffffffffu, row, 0);
+      from[i] = row < 0 ? first : row;
+    }
   }
   const unsigned short* src = reinterpret_cast<const unsigned short*>(grp.dY[blockIdx.z]);
   unsigned short* dst = reinterpret_cast<unsigned short*>(grp.Ag[blockIdx.z]) + jb + lane;
@@ -834,7 +841,7 @@ gather_cols_kernel(const GatherGroup grp, long long lddy, int T, int m, int r, i
 #pragma unroll
       for (int i = 0; i < NI; ++i) {
         v[u][i] = 0;
-        if (i < live) v[u][i] = ptx::ld_na_u16<SPARSE>(line + max(rows[i], 0));
+        if (i < live) v[u][i] = ptx::ld_na_u16<SPARSE>(line + max(from[i], 0));
       }
     }
 #pragma unroll
