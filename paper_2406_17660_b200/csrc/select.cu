@@ -11,8 +11,9 @@
 // cluster of eight CTAs, about two rows a thread, that exchange histograms and counts through
 // distributed shared memory: 13824 rows without replacement took 37 us on one CTA, 14 on eight; up to
 // 4096 rows one CTA is as fast for Top-r (10 us at 4096, 12 on a cluster: six cluster barriers).  A score costs a Philox
-// block and an fp64 logarithm, so without replacement the cluster pays from 1025 rows (9.6 us either way there; 2368 rows
-// 11.3 -> 9.6, 4096 rows 13.6 -> 9.7).
+// block and an fp64 logarithm, so without replacement the cluster pays from 2049 rows (us on one CTA and on the cluster, r = m/64
+// to m/2: 1025 rows 7.6 to 8.0 and 8.7 to 8.9, 1900 8.6 to 9.2 and 8.8 to 9.0, 2049 9.4 to 10.3 and 8.9 to 9.1, 4096 12.4 to 13.8 and
+// 9.1 to 9.2).
 // Sampling with replacement is a serial chain (running sum, search, expansion) and stays on one.
 //
 //   Top-r: the fp32 bit pattern of a non-negative float orders like the float,
@@ -497,9 +498,9 @@ int allow_smem(K kernel, bool (&done)[64]) {
   return GRASS_OK;
 }
 
-// Ranking: eight CTAs (the portable cluster size) from 4097 rows up, 1025 where rows are scored, else one.
+// Ranking: eight CTAs (the portable cluster size) from 4097 rows up, 2049 where rows are scored, else one.
 int launch_rank(SelectArgs& a, cudaStream_t s) {
-  const int ctas = a.m > (is_nr(a.method) ? 1 : 4) * kThreads ? 8 : 1;
+  const int ctas = a.m > (is_nr(a.method) ? 2 : 4) * kThreads ? 8 : 1;
   const int rows = static_cast<int>(round_up((static_cast<size_t>(a.m) + ctas - 1) / ctas, 32));
   a.stage_norms = rows * sizeof(float) <= kSelectBudget;
   static bool attr_set[64] = {false};
