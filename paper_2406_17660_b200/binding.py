@@ -6,6 +6,7 @@ stream and raises GrassError on a non-zero status; nothing here computes.
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from ctypes import c_double, c_int, c_int32, c_int64, c_size_t, c_uint32, c_uint64, c_void_p
 
@@ -470,14 +471,17 @@ _SCAN = None
 
 
 def _accepted():
-    """accepted() of the built module (csrc/scan.cpp)."""
+    """accepted() of the module that is built for this torch and this Python (csrc/scan.cpp)."""
     global _SCAN
     if _SCAN is None:
-        try:
-            from ._scan import accepted
-        except ImportError as e:
-            raise RuntimeError("the _scan module is missing: build it with `python -m paper_2406_17660_b200.build`") from e
-        _SCAN = accepted
+        from .build import scan_path
+        path = scan_path()
+        if not os.path.exists(path):
+            raise RuntimeError(f"{path} is missing: build it with `python -m paper_2406_17660_b200.build`")
+        spec = importlib.util.spec_from_file_location(f"{__package__}._scan", path)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        _SCAN = module.accepted
     return _SCAN
 
 

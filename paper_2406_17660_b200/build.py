@@ -2,9 +2,9 @@
 
     python -m paper_2406_17660_b200.build
 
-Produces libgrass_b200.so (the CUDA library, nvcc) and _scan.so (the binding's scan of torch tensors,
-g++ against torch's headers) next to this file.  nvcc cross-compiles without a GPU, so this runs on any
-box with the CUDA toolkit.
+Produces libgrass_b200.so (the CUDA library, nvcc) and the binding's scan of torch tensors (g++ against
+torch's and Python's headers, whose object layouts it is built for: its file name carries both versions)
+next to this file.  nvcc cross-compiles without a GPU, so this runs on any box with the CUDA toolkit.
 """
 from __future__ import annotations
 
@@ -18,7 +18,6 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libgrass_b200.so")
-SCAN = os.path.join(HERE, "_scan.so")
 SOURCES = ["common.cu", "row_norms.cu", "select.cu", "project.cu", "adam.cu", "scatter.cu",
            "adam_scatter.cu", "selftest.cu"]
 
@@ -30,10 +29,17 @@ def _nvcc() -> str:
     raise RuntimeError("nvcc not found; set NVCC or install the CUDA toolkit")
 
 
+def scan_path() -> str:
+    """The scan module for the torch and the Python that run now."""
+    import torch
+    return os.path.join(HERE, f"_scan.{sysconfig.get_config_var('SOABI')}.torch-{torch.__version__}.so")
+
+
 def _stale() -> bool:
-    if not (os.path.exists(LIB) and os.path.exists(SCAN)):
+    scan = scan_path()
+    if not (os.path.exists(LIB) and os.path.exists(scan)):
         return True
-    t = min(os.path.getmtime(LIB), os.path.getmtime(SCAN))
+    t = min(os.path.getmtime(LIB), os.path.getmtime(scan))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)]
     deps += [os.path.join(ROOT, "include", f) for f in os.listdir(os.path.join(ROOT, "include"))]
     return any(os.path.getmtime(d) > t for d in deps)
@@ -46,8 +52,9 @@ def _scan_command() -> list:
            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
     for path in include_paths():
         cmd += ["-isystem", path]
-    return cmd + ["-I", sysconfig.get_paths()["include"], "-o", SCAN, os.path.join(CSRC, "scan.cpp"), "-L",
-                  os.path.join(os.path.dirname(torch.__file__), "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10"]
+    return cmd + ["-I", sysconfig.get_paths()["include"], "-I", os.path.join(ROOT, "include"), "-o", scan_path(),
+                  os.path.join(CSRC, "scan.cpp"), "-L", os.path.join(os.path.dirname(torch.__file__), "lib"),
+                  "-ltorch_python", "-ltorch_cpu", "-lc10"]
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -67,7 +74,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     res = subprocess.run(_scan_command(), capture_output=True, text=True)
     if res.returncode != 0:
         sys.stderr.write(res.stdout + res.stderr)
-        raise RuntimeError("g++ failed building _scan.so")
+        raise RuntimeError("g++ failed building the scan module")
     return LIB
 
 

@@ -8,8 +8,11 @@
 #include <Python.h>
 #include <torch/csrc/autograd/python_variable.h>
 
+#include <cstddef>
 #include <cstdint>
 #include <cstring>
+
+#include "grass.h"
 
 namespace {
 
@@ -18,6 +21,10 @@ struct Seen {
   int64_t dtype, device, dim, numel, contiguous, sizes[2], strides[2];
 };
 constexpr int kMost = 8;
+// bytes from a layer's pointer in one of grass_step_t's arrays to its pointer in the next
+constexpr std::size_t kField = offsetof(grass_step_t, X) - offsetof(grass_step_t, dY);
+static_assert(kField == GRASS_MAX_GROUP * sizeof(void*) && offsetof(grass_step_t, W) == offsetof(grass_step_t, dY) + 8 * kField,
+              "nine arrays of GRASS_MAX_GROUP pointers, one after the other");
 
 // False: not a plain tensor that has storage (the caller's own checks decide).
 bool look(PyObject* o, Seen& s, void*& at) {
@@ -41,7 +48,7 @@ bool look(PyObject* o, Seen& s, void*& at) {
   return true;
 }
 
-// accepted(address, before, tensor or None, ...): True, and tensor i's address is at address + 64 i, if the tensors are
+// accepted(address, before, tensor or None, ...): True, and tensor i's address is at address + i kField, if the tensors are
 // alike in all but their addresses to those that `before` describes; else their description, or None where there is none.
 PyObject* accepted(PyObject*, PyObject* const* args, Py_ssize_t n) {
   if (n < 3 || n - 2 > kMost) {
@@ -64,7 +71,7 @@ PyObject* accepted(PyObject*, PyObject* const* args, Py_ssize_t n) {
   PyObject* before = args[1];
   if (PyBytes_Check(before) && PyBytes_GET_SIZE(before) == bytes &&
       std::memcmp(PyBytes_AS_STRING(before), now, bytes) == 0) {
-    for (Py_ssize_t i = 0; i < count; ++i) *reinterpret_cast<void**>(address + 64 * i) = at[i];
+    for (Py_ssize_t i = 0; i < count; ++i) *reinterpret_cast<void**>(address + kField * i) = at[i];
     Py_RETURN_TRUE;
   }
   return PyBytes_FromStringAndSize(now, bytes);
