@@ -51,11 +51,13 @@ struct ProfileScope {
 // call or of the stream writes, so completion is transitive along the chain and along the stream.  There is no exception for
 // what a kernel further back wrote: the wait makes visible what the grids before it wrote, and nothing is said of a
 // read ahead of it.  (An update that read M, V, W and idx before its wait took 10.7 us instead of 11.3 a step of
-// T = 2048, 512 x 512, r = 128, 170.0 instead of 171.5 of T = 4096, 5120 x 13824, r = 1024.)  The kernel that another
-// call's first kernel follows lets it in only by ending.  Eagerly launched steps gained 1 to 2.7 us from the
-// attribute on their first kernel (T = 4096, 1024 x 1024, r = 128: 16.4 -> 13.7).
-// A kernel that something follows in its call lets it in with grid_dep_launch(), late enough that the waiting
-// blocks do not hold an SM that another stream could use.
+// T = 2048, 512 x 512, r = 128, 170.0 instead of 171.5 of T = 4096, 5120 x 13824, r = 1024.)  Eagerly launched steps gained 1
+// to 2.7 us from the attribute on their first kernel (T = 4096, 1024 x 1024, r = 128: 16.4 -> 13.7).
+// A kernel that something may follow in its call lets it in with grid_dep_launch(), late enough that what is left is short.
+// It does so too where it is its call's last (selections, row norms, an unsplit projection), so the next call's first kernel
+// may be resident while this one still writes, and a projection then holds its SMs.  Another stream does not miss them: 60 x
+// (selection of 13824 rows, projection of T = 4096) beside 60 steps of 1B down take 5.49 ms, and 5.61 if last
+// kernels let nothing in; refreshes of 60M, 350M, 1B and 7B layers on two streams take 0 to 3 % longer so.
 // What an earlier kernel writes (inputs made by the program's last kernel, G_C, partials, norms, idx, rho, the gathered
 // operand) is still being written when a dependent kernel becomes resident, so it is not constant for that kernel's
 // lifetime: such a kernel reads it with ordinary loads (also ptx::ld_s32, ld_f32, ld_na_u16), through pointers

@@ -195,6 +195,7 @@ TileCost tile_cost(const Problem& q, const TileChoice& t) {
   k.hbm = x_mb / 6.0;
   k.gather = k.around = 0;
   if (t.gather == kOptPrepass) {
+    // (fitted to a gather with fewer loads in flight: too dear by 1.3 to 1.6 at 512 x 512, r = 128)
     k.hbm += 1.1 * ag_mb / 6.0;
     k.around = 0.5 + pow(pow_2_5(lsu * (0.87 + 0.033 * per_load)) + pow_2_5((dy_mb + ag_mb) / 6.6), 0.4);
   } else if (t.gather == kOptCoop) {
@@ -789,6 +790,7 @@ size_t grad_parts_bytes(int split_k, int64_t m, long long ld) {
 // 256 .. 5461, T = 256 .. 65536, r = 8 .. 1024).  Over these it costs 0.3 % more than the better form,
 // always keeping 25 %, never 21 %; weighing the partials' bytes alone against the projection cost 0.8 %, and up to
 // 50 % where few rows of a small layer make many slices (T = 13056, 384 x 5461, r = 43: kept 155 us, projected 113).
+// (Since the norms leave the partials' sum for the update, keeping costs up to 10 % less than in that fit.)
 bool make_keep_plan(int64_t T, int64_t m, int64_t n, int r, TcPlan* plan) {
   bool small = false;
   const double norms_us = make_norms_plan(T, m, n, &small).us;

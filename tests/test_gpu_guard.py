@@ -71,7 +71,7 @@ def test_row_norms_stays_inside_norms(m, n, ld, dtype):
 
 
 @pytest.mark.parametrize("method", [grass.SEL_TOPR, grass.SEL_MULTINOMIAL_NORM, grass.SEL_UNIFORM_NR])
-@pytest.mark.parametrize("m,r", [(300, 1), (300, 300), (13824, 1024), (16384, 77)])
+@pytest.mark.parametrize("m,r", [(300, 1), (300, 300), (2049, 2049), (2305, 100), (13824, 1024), (16384, 77)])
 def test_select_stays_inside_idx_rho_and_workspace(method, m, r):
     lam = torch.rand(m, device=DEV) + 0.1
     for static in (False, True):
